@@ -23,6 +23,7 @@ struct qpr_ctx {
     int np = 0;
     double alpha = 0.0, omega = 0.0;
     qpr_options opt{};
+    int nnz = 0;           // entries of H
     double spread = 0.0;   // estimated lambda_max - lambda_min of H
     double cmax = 1.0;     // max column sum of G
     // device operators
@@ -215,7 +216,18 @@ qpr_status run_rk4(qpr_ctx *ctx, double dt, double tol, int64_t max_steps) {
     h->dt = dt;
     h->scale = 1.0;
     QPR_CUDA(ctx, cudaMemcpyAsync(ctx->d_ctl, h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream));
-    qpr_status st = ensure_graph(ctx);
+    qpr_status st;
+    if (ctx->n <= qpr::kSmallMaxN) {
+        for (;;) {
+            QPR_CUDA(ctx, qpr::launch_small_rk4(ctx->ops, ctx->work, ctx->nnz, qpr::kSmallSteps, ctx->stream));
+            ctx->launches += 1;
+            QPR_CUDA(ctx, cudaMemcpyAsync(h, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
+            st = sync_ctx(ctx);
+            if (st != QPR_OK) return st;
+            if (h->done) return QPR_OK;
+        }
+    }
+    st = ensure_graph(ctx);
     if (st != QPR_OK) return st;
     const int chunk = ctx->graph ? ctx->graph_steps : 1;
     // Each stage-2 gain kernel stops the run once max_steps is reached, so
@@ -828,6 +840,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
                     (o.backend == QPR_BACKEND_DENSE ||
                      (o.backend == QPR_BACKEND_AUTO && (double)hval.size() >= (double)n * (double)n / 8.0));
     if (tc) ctx->np = (int)(((n + qpr::kTileTc - 1) / qpr::kTileTc) * qpr::kTileTc);
+    ctx->nnz = (int)hval.size();
     ctx->spread = qpr::estimate_spread(n, hptr, hcol, hval);
     if (o.backend == QPR_BACKEND_AUTO)
         ctx->backend = ((double)hval.size() < (double)n * (double)n / 8.0) ? QPR_BACKEND_SPARSE : QPR_BACKEND_DENSE;
@@ -862,6 +875,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     CREATE_CUDA(qpr::init_stage_fp64());
     CREATE_CUDA(qpr::init_stage_sparse());
     CREATE_CUDA(qpr::init_stage_mixed());
+    if (n <= qpr::kSmallMaxN) CREATE_CUDA(qpr::init_small((int)n, ctx->nnz));
     const int np = ctx->np;
     const size_t plane = (size_t)np * np;
     // dense H, np x np with zero padding

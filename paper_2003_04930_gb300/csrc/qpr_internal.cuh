@@ -236,6 +236,17 @@ cudaError_t init_stage_fp64();
 void launch_stage_sparse(int stage, const DevOps &ops, const Work &w, cudaStream_t s);
 cudaError_t init_stage_sparse();
 
+// ---- FP64 RK4 of a small problem, one cluster, many steps a launch (stage_small.cu) ----
+// Up to `limit` steps from the state in w.y, or until the stop rule sets
+// ctl->done; nnz: the entries of H. One launch is at most kSmallSteps steps
+// (40 ms at the largest N). The line at 44: the last size with an octet of
+// lanes per element in one cluster's warps; at 45 the eight launches take 366
+// us a step, at 44 this form 39.
+constexpr int kSmallMaxN = 44;
+constexpr int kSmallSteps = 1024;
+cudaError_t init_small(int n, int nnz);
+cudaError_t launch_small_rk4(const DevOps &ops, const Work &w, int nnz, int limit, cudaStream_t s);
+
 // ---- mixed-precision form (stage_mixed.cu) ----
 // Reference refresh: R = y = y / tr(y), F = f(R) exactly (FP64), D = 0, exact
 // residual and stop decision.
