@@ -59,7 +59,7 @@ gain_kernel(DevOps ops, Work w, const double *__restrict__ yin) {
     if (threadIdx.x == 0) s_done = *(volatile int *)&w.ctl->done;
     __syncthreads();
     if (s_done) return;
-    gain64::gain_fp64_body<STAGE>(ops, w, yin, blockIdx.x, gridDim.x);
+    gain64::gain_fp64_body(STAGE, ops, w, yin, (size_t)ops.np + 1, blockIdx.x, gridDim.x);
 }
 
 int grid_for(size_t work, int threads) {

@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(256) b_gain64_kernel(const BatchGraph *gs, con
     __shared__ int s_flag;
     load_graph(gs, act[blockIdx.x], sg);
     if (skip_refresh(sg, act[blockIdx.x], due, &s_flag)) return;
-    gain64::gain_fp64_body<0>(sg.ops, sg.w64, sg.w64.y, 0, 1);
+    gain64::gain_fp64_body(0, sg.ops, sg.w64, sg.w64.y, (size_t)sg.ops.np + 1, 0, 1);
 }
 
 __global__ void __launch_bounds__(sparse64::NTHREADS)

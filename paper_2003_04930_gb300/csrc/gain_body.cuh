@@ -14,42 +14,59 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Fixed-order block sum, broadcast to every thread (blockDim.x <= 1024).
-__device__ __forceinline__ double block_sum(double v, double *red) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// The threads that work together: a whole CTA, or its warps from `FIRST` on
+// (synchronised by barrier 1).
+struct Cta {
+    __device__ __forceinline__ int tid() const { return threadIdx.x; }
+    __device__ __forceinline__ int size() const { return blockDim.x; }
+    __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
+template <int FIRST, int THREADS>
+struct Warps {
+    __device__ __forceinline__ int tid() const { return threadIdx.x - 32 * FIRST; }
+    __device__ __forceinline__ int size() const { return THREADS; }
+    __device__ __forceinline__ void sync() const { asm volatile("bar.sync 1, %0;\n" ::"n"(THREADS) : "memory"); }
+};
+
+// Fixed-order sum over the group, broadcast to every thread (1024 at most).
+template <typename G = Cta>
+__device__ __forceinline__ double block_sum(double v, double *red, G grp = G{}) {
+    const int lane = threadIdx.x & 31, warp = grp.tid() >> 5;
     v = warp_sum(v);
-    __syncthreads();  // red may still be read by a previous call
+    grp.sync();  // red may still be read by a previous call
     if (lane == 0) red[warp] = v;
-    __syncthreads();
+    grp.sync();
     double s = 0.0;
-    const int nw = (blockDim.x + 31) >> 5;
+    const int nw = (grp.size() + 31) >> 5;
     for (int q = 0; q < nw; ++q) s += red[q];
     return s;
 }
 
-// g = G p with G = alpha S + (1 - alpha) F (Eq. S2, Eq. S4), p_j = sig Y_jj:
+// g = G p with G = alpha S + (1 - alpha) F (Eq. S2, Eq. S4), p_j = Y_jj
+// (diag[j stride]):
 //   (S p)_i = sum_{j with out-links} A_ij / outDeg(j) p_j  +  dangling part,
 //   dangling part = (D - [i dangles] p_i) / (N - 1)  (F columns)  or  D / N,
 //   (F p)_i = (P - p_i) / (N - 1),
 // with P = sum_j p_j and D = sum over dangling j of p_j.
-// Stage 1 also fixes sig = 1 / Re tr(y) for the whole step. Stage 2 first
-// reduces the residual partials of stage 1 into ||f(y_n)||_F and takes the
-// stop decision (one CTA).
-// blk / nblk: this CTA's index and the number of CTAs sharing the rows; the
+// Stage 1 also publishes 1 / Re tr(y), by which stage 4 normalises the step.
+// Stage 2 first reduces the residual partials of stage 1 into ||f(y_n)||_F of
+// the normalised state and takes the stop decision (one CTA).
+// blk / nblk: this group's index and the number of groups sharing the rows; the
 // residual decision (stage 2) is taken by blk 0.
-template <int STAGE>
-__device__ __forceinline__ void gain_fp64_body(const DevOps &ops, const Work &w, const double *__restrict__ yin,
-                                               int blk, int nblk) {
+template <typename G = Cta>
+__device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, const Work &w,
+                                               const double *__restrict__ diag, size_t stride, int blk, int nblk,
+                                               G grp = G{}) {
     __shared__ double red[32];
     Ctl *ctl = w.ctl;
     const int n = ops.n, np = ops.np;
 
-    if (STAGE == 2 && blk == 0) {
+    if (stage == 2 && blk == 0) {
         double s = 0.0;
-        for (int i = threadIdx.x; i < w.npairs; i += blockDim.x) s += w.partials[i];
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) {
-            const double r = sqrt(s);
+        for (int i = grp.tid(); i < w.npairs; i += grp.size()) s += w.partials[i];
+        s = block_sum(s, red, grp);
+        if (grp.tid() == 0) {
+            const double r = ctl->scale * sqrt(s);
             ctl->resid = r;
             ctl->resid_step = ctl->step;
             if (!isfinite(r)) {
@@ -65,48 +82,48 @@ __device__ __forceinline__ void gain_fp64_body(const DevOps &ops, const Work &w,
         }
     }
 
+    // independent of the sums below: the reciprocal, and the row sum of this
+    // warp's first row, whose loads then fly with those of the diagonal
+    const double inv_nm1 = __drcp_rn((double)(n - 1));
+    const int lane = threadIdx.x & 31;
+    const int wpb = grp.size() >> 5;
+    const int first = blk * wpb + (grp.tid() >> 5);
+    auto row_part = [&](int i) {
+        double s = 0.0;
+        if (i < n) {
+            for (int q = ops.s_ptr[i] + lane; q < ops.s_ptr[i + 1]; q += 32)
+                s = __fma_rn(ops.s_val[q], diag[ops.s_col[q] * stride], s);
+        }
+        return s;
+    };
+    double s0 = row_part(first);
     double P = 0.0, D = 0.0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const double pj = yin[(size_t)j * np + j];
+    for (int j = grp.tid(); j < n; j += grp.size()) {
+        const double pj = diag[j * stride];
         P += pj;
         if (ops.dang[j]) D += pj;
     }
-    P = block_sum(P, red);
-    D = block_sum(D, red);
-    double sig = 1.0;
-    if (STAGE == 1) {
-        sig = 1.0 / P;
-        if (blk == 0 && threadIdx.x == 0) {
-            ctl->scale = sig;
-            ctl->trace = P;
-            if (!(P > 0.0) || !isfinite(P)) {
-                ctl->status = kCtlNonFinite;
-                ctl->done = 1;
-            }
+    P = block_sum(P, red, grp);
+    D = block_sum(D, red, grp);
+    if (stage == 1 && blk == 0 && grp.tid() == 0) {
+        ctl->scale = 1.0 / P;
+        ctl->trace = P;
+        if (!(P > 0.0) || !isfinite(P)) {
+            ctl->status = kCtlNonFinite;
+            ctl->done = 1;
         }
     }
-    const double Ps = __dmul_rn(sig, P), Ds = __dmul_rn(sig, D);
-    const double inv_nm1 = __drcp_rn((double)(n - 1));
-    const int lane = threadIdx.x & 31;
-    const int wpb = blockDim.x >> 5;
-    for (int i = blk * wpb + (threadIdx.x >> 5); i < np; i += nblk * wpb) {
-        double s = 0.0;
-        if (i < n) {
-            for (int q = ops.s_ptr[i] + lane; q < ops.s_ptr[i + 1]; q += 32) {
-                const int j = ops.s_col[q];
-                s = __fma_rn(ops.s_val[q], __dmul_rn(sig, yin[(size_t)j * np + j]), s);
-            }
-        }
-        s = warp_sum(s);
+    for (int i = first; i < np; i += nblk * wpb) {
+        const double s = warp_sum(i == first ? s0 : row_part(i));
         if (lane == 0) {
             double gi = 0.0;
             if (i < n) {
-                const double pi = __dmul_rn(sig, yin[(size_t)i * np + i]);
+                const double pi = diag[i * stride];
                 const double dterm = (ops.dangling == QPR_DANGLING_F)
-                                         ? __dmul_rn(__dsub_rn(Ds, ops.dang[i] ? pi : 0.0), inv_nm1)
-                                         : __ddiv_rn(Ds, (double)n);
+                                         ? __dmul_rn(__dsub_rn(D, ops.dang[i] ? pi : 0.0), inv_nm1)
+                                         : __ddiv_rn(D, (double)n);
                 gi = __fma_rn(ops.alpha, __dadd_rn(s, dterm),
-                              __dmul_rn(__dmul_rn(__dsub_rn(1.0, ops.alpha), __dsub_rn(Ps, pi)), inv_nm1));
+                              __dmul_rn(__dmul_rn(__dsub_rn(1.0, ops.alpha), __dsub_rn(P, pi)), inv_nm1));
             }
             w.g[i] = gi;
         }

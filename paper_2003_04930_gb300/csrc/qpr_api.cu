@@ -46,6 +46,11 @@ struct qpr_ctx {
     __nv_bfloat16 *d_dsplit = nullptr;  // dense mixed form: 3 delta-split buffers of 6 planes
     int2 *d_pairs_tc = nullptr;
     qpr::TcMaps tcmaps{};
+    void *d_digits = nullptr;   // FP64 dense form on the tensor cores: digit planes, exponents, X
+    int *d_digint = nullptr;
+    double *d_digx = nullptr;
+    qpr::DigitWork digits{};
+    qpr::DigitMaps digitmaps{};
     int2 *d_colkh = nullptr;    // column-block form: packed CSR, plan arrays, X = H delta
     int *d_colint = nullptr;    // q | sb | wb
     int4 *d_colpieces = nullptr;
@@ -134,7 +139,8 @@ qpr_status sync_ctx(qpr_ctx *ctx) {
 }
 
 void launch_stage(qpr_ctx *ctx, int s) {
-    if (ctx->backend == QPR_BACKEND_DENSE) qpr::launch_stage_fp64(s, ctx->ops, ctx->work, ctx->stream);
+    if (ctx->d_digits) qpr::launch_stage_digits(s, ctx->ops, ctx->work, ctx->digits, ctx->digitmaps, ctx->stream);
+    else if (ctx->backend == QPR_BACKEND_DENSE) qpr::launch_stage_fp64(s, ctx->ops, ctx->work, ctx->stream);
     else qpr::launch_stage_sparse(s, ctx->ops, ctx->work, ctx->stream);
 }
 
@@ -142,10 +148,12 @@ void enqueue_step(qpr_ctx *ctx) {
     const qpr::Work &w = ctx->work;
     const double *yin[5] = {w.y, w.y, w.ya, w.yb, w.ya};
     for (int s = 1; s <= 4; ++s) {
-        qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream);
+        if (!ctx->d_digits) qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream);
         launch_stage(ctx, s);
     }
 }
+
+int fp64_launches_per_step(const qpr_ctx *ctx) { return 4 * (ctx->d_digits ? qpr::kDigitLaunches : 2); }
 
 qpr_status ensure_graph(qpr_ctx *ctx) {
     if (ctx->graph || ctx->opt.graph_steps <= 0) return QPR_OK;
@@ -238,10 +246,11 @@ qpr_status run_rk4(qpr_ctx *ctx, double dt, double tol, int64_t max_steps) {
         } else {
             enqueue_step(ctx);
         }
-        ctx->launches += 8 * (int64_t)chunk;
+        ctx->launches += fp64_launches_per_step(ctx) * (int64_t)chunk;
         QPR_CUDA(ctx, cudaMemcpyAsync(h, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
         st = sync_ctx(ctx);
         if (st != QPR_OK) return st;
+        if (h->err_timeout) return fail(ctx, QPR_E_TIMEOUT, "a device-side wait gave up (err_timeout set by a stage kernel)");
         if (h->done) break;
     }
     return QPR_OK;
@@ -743,6 +752,9 @@ void qpr_destroy(qpr_ctx *ctx) {
     if (ctx->graph_rkf) cudaGraphExecDestroy(ctx->graph_rkf);
     cudaFree(ctx->d_rkf);
     cudaFree(ctx->d_H);
+    cudaFree(ctx->d_digits);
+    cudaFree(ctx->d_digint);
+    cudaFree(ctx->d_digx);
     cudaFree(ctx->d_hptr);
     cudaFree(ctx->d_rowseg);
     cudaFree(ctx->d_seg);
@@ -878,14 +890,6 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     if (n <= qpr::kSmallMaxN) CREATE_CUDA(qpr::init_small((int)n, ctx->nnz));
     const int np = ctx->np;
     const size_t plane = (size_t)np * np;
-    // dense H, np x np with zero padding
-    {
-        std::vector<double> Hd(plane, 0.0);
-        for (int64_t i = 0; i < n; ++i)
-            for (int64_t q = hptr[i]; q < hptr[i + 1]; ++q) Hd[(size_t)i * np + hcol[q]] = hval[q];
-        CREATE_CUDA(cudaMalloc(&ctx->d_H, plane * sizeof(double)));
-        CREATE_CUDA(cudaMemcpy(ctx->d_H, Hd.data(), plane * sizeof(double), cudaMemcpyHostToDevice));
-    }
     {
         std::vector<int> hptr32(n + 1);
         for (int64_t i = 0; i <= n; ++i) hptr32[i] = (int)hptr[i];
@@ -1115,6 +1119,44 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     wk.npairs = (int)pairs.size();
     wk.tiles = T;
     wk.ctl = ctx->d_ctl;
+    if (o.precision == QPR_FP64 && ctx->backend == QPR_BACKEND_DENSE) {
+        // the product on the tensor cores by exact digits where a plan keeps
+        // the sums exact and its planes fit beside everything else; else the
+        // FP64 tensor kernel and its dense H (N = 500, unit weights: 616 us a
+        // stage there, 27 us here; N = 922, lognormal weights: 4.2 and 0.36 ms)
+        qpr::DigitPlan dplan;
+        bool digits = qpr::plan_digits(hops, dplan);
+        if (digits) {
+            cudaError_t e = cudaMalloc(&ctx->d_digits, qpr::digits_half_count(dplan, np) * 2);
+            if (e == cudaSuccess) e = cudaMalloc(&ctx->d_digint, 3 * (size_t)np * sizeof(int));
+            if (e == cudaSuccess) e = cudaMalloc(&ctx->d_digx, 2 * plane * sizeof(double));
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                cudaFree(ctx->d_digits);
+                cudaFree(ctx->d_digint);
+                ctx->d_digits = nullptr;
+                ctx->d_digint = nullptr;
+                digits = false;
+            } else if (e != cudaSuccess) {
+                return bail(cuda_fail(ctx, e, "cudaMalloc"));
+            }
+        }
+        cudaError_t e = cudaSuccess;
+        if (digits) {
+            int sms = 0;
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+            e = qpr::init_digits(ops, dplan, sms, ctx->d_digits, ctx->d_digint, ctx->d_digx, &ctx->digits, &ctx->digitmaps);
+        } else {
+            // dense H, np x np with zero padding
+            std::vector<double> Hd(plane, 0.0);
+            for (int64_t i = 0; i < n; ++i)
+                for (int64_t q = hptr[i]; q < hptr[i + 1]; ++q) Hd[(size_t)i * np + hcol[q]] = hval[q];
+            e = cudaMalloc(&ctx->d_H, plane * sizeof(double));
+            if (e == cudaSuccess) e = cudaMemcpy(ctx->d_H, Hd.data(), plane * sizeof(double), cudaMemcpyHostToDevice);
+            ops.H = ctx->d_H;
+        }
+        if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "dense operator"));
+    }
     if (o.precision == QPR_MIXED) {
         qpr::MixedWork &mw = ctx->mw;
         mw.R = ctx->d_mix64;
@@ -1223,18 +1265,21 @@ static qpr_status rhs_impl(qpr_ctx *ctx, const void *rho, void *out, double *res
     memset(h, 0, sizeof(Ctl));
     h->scale = 1.0;
     QPR_CUDA(ctx, cudaMemcpyAsync(ctx->d_ctl, h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream));
-    qpr::launch_gain(0, ctx->ops, ctx->work.y, ctx->work, ctx->stream);
+    if (!ctx->d_digits) qpr::launch_gain(0, ctx->ops, ctx->work.y, ctx->work, ctx->stream);
     launch_stage(ctx, 0);
     if (out) {
         st = export_rho(ctx, ctx->work.z, 0, out);
         if (st != QPR_OK) return st;
     }
+    if (ctx->d_digits)
+        QPR_CUDA(ctx, cudaMemcpyAsync(h, ctx->d_ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, ctx->stream));
     std::vector<double> part(ctx->work.npairs);
     if (resid)
         QPR_CUDA(ctx, cudaMemcpyAsync(part.data(), ctx->d_partials, part.size() * sizeof(double),
                                       cudaMemcpyDeviceToHost, ctx->stream));
     st = sync_ctx(ctx);
     if (st != QPR_OK) return st;
+    if (h->err_timeout) return fail(ctx, QPR_E_TIMEOUT, "a device-side wait gave up (err_timeout set by a stage kernel)");
     if (resid) {
         double s = 0.0;
         for (double v : part) s += v;

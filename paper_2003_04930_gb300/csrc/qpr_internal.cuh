@@ -232,6 +232,40 @@ void launch_stage_fp64(int stage, const DevOps &ops, const Work &w, cudaStream_t
 // Opt in to the kernel's dynamic shared memory on the current device.
 cudaError_t init_stage_fp64();
 
+// ---- FP64 dense stage on the tensor cores (stage_digits.cu), same contract ----
+// Plan: b bits per digit, s digits of every row of Y, sh of H; erow: per row
+// of H the binary exponent of its first digit's unit.
+struct HostOps;
+struct DigitPlan {
+    int b = 0, s = 0, sh = 0;
+    std::vector<int> erow;
+};
+struct DigitWork {
+    int b, s, sh;
+    int ring_a, ring_b;   // pipeline depths: digit planes of H, blocks of Y
+    int gain_ctas;        // leading CTAs of the product launch that form the gain beside their tile
+    unsigned tmem_cols;
+    int epi_smem;         // dynamic shared memory of the epilogue
+    void *yd;             // FP16 digits of the stage input [s][2 planes][np][np]
+    int *ecol;            // [2 planes][np]: the exponent of the first digit's unit of a row of Y
+    int *erow;            // np
+    double *x;            // [H Re Y ; -H Im Y], 2 planes
+};
+struct DigitMaps {
+    CUtensorMap h, y;
+};
+// False if no digit width keeps the sums exact (stage_fp64.cu serves then).
+bool plan_digits(const HostOps &h, DigitPlan &p);
+// FP16 values of the digit planes; ints: 3 np, x: 2 np^2.
+size_t digits_half_count(const DigitPlan &p, int np);
+cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *halves, int *ints, double *x, DigitWork *dw,
+                        DigitMaps *maps);
+// The whole stage: digits of its input, product (with the gain and, at stage
+// 2, the stop decision), epilogue.
+void launch_stage_digits(int stage, const DevOps &ops, const Work &w, const DigitWork &d, const DigitMaps &m,
+                         cudaStream_t s);
+constexpr int kDigitLaunches = 3;
+
 // ---- sparse (CSR H) FP64 stage kernel (stage_sparse.cu), same contract ----
 void launch_stage_sparse(int stage, const DevOps &ops, const Work &w, cudaStream_t s);
 cudaError_t init_stage_sparse();

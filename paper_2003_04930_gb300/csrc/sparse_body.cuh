@@ -9,10 +9,9 @@ namespace qpr {
 namespace sparse64 {
 
 constexpr int TS = kEpiTS;
-constexpr int NTHREADS = kEpiThreads;
+constexpr int NTHREADS = 256;
 constexpr int LDX = 2 * TS + 1;
-constexpr int LDO = kEpiLDO;
-constexpr int SMEM_BYTES = (2 * TS * LDX + 4 * TS * LDO) * (int)sizeof(double);
+constexpr int SMEM_BYTES = 2 * TS * LDX * (int)sizeof(double);
 
 // rows `rowtile` of H times columns `coltile` of Y into sX ([TS][LDX]).
 __device__ __forceinline__ void spmm_tile(const DevOps &ops, const double *__restrict__ yin, size_t plane,
@@ -65,11 +64,12 @@ __device__ __forceinline__ void tile(const DevOps &ops, const Work &w, int I, in
     const double *__restrict__ yin = (STAGE <= 1) ? w.y : (STAGE == 3 ? w.yb : w.ya);
     double *sX1 = smem;
     double *sX2 = smem + TS * LDX;
-    double *sO = smem + 2 * TS * LDX;
+    EpiIn<STAGE, NTHREADS> in;
     spmm_tile(ops, yin, plane, I, J, sX1);
     if (!diag) spmm_tile(ops, yin, plane, J, I, sX2);
+    in.load(ops, w, I, J);  // after the product: its registers are free (725 -> 615 us a step at N = 922)
     __syncthreads();
-    stage_epilogue<STAGE>(ops, w, I, J, diag, sX1, sX2, LDX, sO, red, pidx, first);
+    stage_epilogue<STAGE, NTHREADS>(ops, w, I, J, diag, in, sX1, sX2, LDX, red, pidx, first);
     __syncthreads();
 }
 

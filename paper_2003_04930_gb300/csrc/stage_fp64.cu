@@ -16,13 +16,8 @@
 //     X_IJ(a, b) = sum_k H(a, k) Re Y(b, k) - i sum_k H(a, k) Im Y(b, k),
 // since Re Y(k, b) = Re Y(b, k) and Im Y(k, b) = -Im Y(b, k).
 //
-// Classical RK4 (Supplementary Note 2): with Y1 = y / tr(y)
-//   stage 1: k1 = f(Y1); Z = Y1 + dt/6 k1; Ya = Y1 + dt/2 k1 (and ||k1||^2)
-//   stage 2: k2 = f(Ya); Z += dt/3 k2;     Yb = Y1 + dt/2 k2
-//   stage 3: k3 = f(Yb); Z += dt/3 k3;     Ya = Y1 + dt k3
-//   stage 4: k4 = f(Ya); y = Z + dt/6 k4
-// Stage 1 reads the unnormalised y and multiplies by 1/tr(y) in the
-// epilogue (f is linear), which is the per-step trace renormalisation.
+// The RK4 step is the nested form of stage_epilogue.cuh. This kernel serves
+// the weights for which stage_digits.cu has no plan of exact digits.
 //
 // The FP64 tensor path is mma.sync m8n8k4 (DMMA): tcgen05 has no f64 kind.
 #include "qpr_internal.cuh"
@@ -39,11 +34,10 @@ constexpr int NPANEL = 6;              // H_I, ReY_I, ImY_I, H_J, ReY_J, ImY_J
 constexpr int STAGE_DBL = NPANEL * PANEL;
 constexpr int SMEM_BYTES = 2 * STAGE_DBL * (int)sizeof(double);
 constexpr int LDX = 2 * TS + 1;        // epilogue X tile row (odd: conflict-free transpose)
-constexpr int LDO = TS + 1;
 constexpr int NTHREADS = 128;
 
-static_assert(TS == kEpiTS && NTHREADS == kEpiThreads && LDO == kEpiLDO, "epilogue geometry");
-static_assert(2 * TS * LDX + 4 * TS * LDO <= 2 * STAGE_DBL, "epilogue must fit in the pipeline buffers");
+static_assert(TS == kEpiTS, "epilogue geometry");
+static_assert(2 * TS * LDX <= 2 * STAGE_DBL, "epilogue must fit in the pipeline buffers");
 
 __device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
     unsigned s = (unsigned)__cvta_generic_to_shared(smem);
@@ -156,7 +150,8 @@ stage_fp64_kernel(DevOps ops, Work w) {
     // ---- epilogue ----
     double *sX1 = smem;                 // X_IJ: [TS][LDX], columns 0..TS-1 real, TS..2TS-1 imaginary
     double *sX2 = smem + TS * LDX;      // X_JI
-    double *sO = smem + 2 * TS * LDX;   // outputs of tile (I, J) kept for the mirrored write
+    EpiIn<STAGE, NTHREADS> in;
+    in.load(ops, w, I, J);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
@@ -170,7 +165,7 @@ stage_fp64_kernel(DevOps ops, Work w) {
             }
     __syncthreads();
     __shared__ double red[NTHREADS / 32];
-    stage_epilogue<STAGE>(ops, w, I, J, diag, sX1, sX2, LDX, sO, red, blockIdx.x, blockIdx.x == 0);
+    stage_epilogue<STAGE, NTHREADS>(ops, w, I, J, diag, in, sX1, sX2, LDX, red, blockIdx.x, blockIdx.x == 0);
 }
 
 template <int STAGE>
