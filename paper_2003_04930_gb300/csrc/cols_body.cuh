@@ -451,11 +451,11 @@ __device__ __forceinline__ void epilogue_load_x(const DevOps &ops, const MixedWo
 
 // The epilogue of pair (I, J) once its X tiles and gain are in shared memory
 // (after a barrier).
-template <int STAGE, bool TICKET = true>
+template <int STAGE, bool TICKET = true, bool SPLIT = false>
 __device__ __forceinline__ void epilogue_pair_staged(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
                                                      bool first, int nparts, const float *sX1, const float *sX2,
                                                      const float *sg, float *sO, const mixed::EpiIn<STAGE, kENT> &in) {
-    mixed::tile_epilogue_in<STAGE, kENT>(ops, w, I, J, pidx, sX1, sX2, sg, sO, in);
+    mixed::tile_epilogue_in<STAGE, kENT, SPLIT>(ops, w, I, J, pidx, sX1, sX2, sg, sO, in);
     if (STAGE == 1 && TICKET) stage1_last_decides(w, nparts);
     if (STAGE == 4 && first && threadIdx.x == 0) w.ctl->step += 1;
 }

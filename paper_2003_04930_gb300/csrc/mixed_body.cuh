@@ -434,14 +434,34 @@ __device__ __forceinline__ void epi_load(const DevOps &ops, const MixedWork &w, 
     in.cb = ops.c32[J * TS + (tid % TS)];  // the column of every element of this thread
 }
 
+__device__ __forceinline__ void split3(float x, __nv_bfloat16 &h0, __nv_bfloat16 &h1, __nv_bfloat16 &h2) {
+    h0 = __float2bfloat16_rn(x);
+    const float r1 = __fsub_rn(x, __bfloat162float(h0));
+    h1 = __float2bfloat16_rn(r1);
+    const float r2 = __fsub_rn(r1, __bfloat162float(h1));
+    h2 = __float2bfloat16_rn(r2);
+}
+
+// The BF16 split of one delta entry (re, im) at offset o of the dense form's
+// B-operand planes [level][plane][row][k]: plane 0 holds Re delta
+// (symmetric), plane 1 -Im delta.
+__device__ __forceinline__ void put_split(__nv_bfloat16 *sp, size_t plane, size_t o, float re, float im) {
+    __nv_bfloat16 r0, r1, r2, i0, i1, i2;
+    split3(re, r0, r1, r2);
+    split3(-im, i0, i1, i2);
+    sp[0 * plane + o] = r0; sp[2 * plane + o] = r1; sp[4 * plane + o] = r2;
+    sp[1 * plane + o] = i0; sp[3 * plane + o] = i1; sp[5 * plane + o] = i2;
+}
+
 // Epilogue of one tile pair (I, J) of stage STAGE from the products
 // sX1 = X_IJ and (unless I == J) sX2 = X_JI of X = H delta, [a][LDX] rows
 // (real part, then imaginary part), and, on a diagonal pair, the gain of
 // its rows in sg, with the operands `in` loaded by epi_load. Writes tile
 // (I, J) and its conjugate mirror (J, I); stage 1 leaves this pair's
 // residual-estimate partial in partials32[pidx]. sO32: 4 * TS * LDO floats
-// of shared memory; NTH threads. Ends with a barrier.
-template <int STAGE, int NTH>
+// of shared memory; NTH threads. SPLIT (dense form): also the BF16 split of
+// the next stage input. Ends with a barrier.
+template <int STAGE, int NTH, bool SPLIT = false>
 __device__ __forceinline__ void tile_epilogue_in(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
                                                  const float *sX1, const float *sX2, const float *sg, float *sO32,
                                                  const EpiIn<STAGE, NTH> &in) {
@@ -450,6 +470,7 @@ __device__ __forceinline__ void tile_epilogue_in(const DevOps &ops, const MixedW
     const int np = ops.np;
     const size_t plane = (size_t)np * np;
     float *dnext = (STAGE == 2) ? w.db : w.da;
+    __nv_bfloat16 *snext = (STAGE == 2) ? w.splitB : (STAGE == 4 ? w.splitD : w.splitA);
     const float *X2 = diag ? sX1 : sX2;
 
     const float om = ops.omega32, cm = __fsub_rn(1.0f, om);
@@ -477,6 +498,7 @@ __device__ __forceinline__ void tile_epilogue_in(const DevOps &ops, const MixedW
             const float Dr = (STAGE == 1) ? dr : in.vr[k], Di = (STAGE == 1) ? di : in.vi[k];
             const float nr = __fmaf_rn(cst, kr, Dr), ni = __fmaf_rn(cst, ki, Di);
             dnext[off] = nr; dnext[plane + off] = ni;
+            if (SPLIT) put_split(snext, plane, off, nr, ni);
             if (ga == gb && w.pv) w.pv[ga] = nr;
             sO32[0 * TS * LDO + a * LDO + b] = nr;
             sO32[1 * TS * LDO + a * LDO + b] = ni;
@@ -486,6 +508,7 @@ __device__ __forceinline__ void tile_epilogue_in(const DevOps &ops, const MixedW
             const ff vi = delta_update(in.vi[k], in.si[k], in.gi[k], in.li[k], dtf, w.ctl->dtl, kdi);
             w.D[off] = vr.hi; w.D[plane + off] = vi.hi;
             w.Dlo[off] = vr.lo; w.Dlo[plane + off] = vi.lo;
+            if (SPLIT) put_split(snext, plane, off, vr.hi, vi.hi);
             if (ga == gb && w.pv) w.pv[ga] = vr.hi;
             sO32[0 * TS * LDO + a * LDO + b] = vr.hi;
             sO32[1 * TS * LDO + a * LDO + b] = vi.hi;
@@ -508,6 +531,8 @@ __device__ __forceinline__ void tile_epilogue_in(const DevOps &ops, const MixedW
         for (int e = tid; e < TS * TS; e += NTH) {
             const int b = e / TS, a = e - (e / TS) * TS;
             const size_t off = (size_t)(J * TS + b) * np + I * TS + a;
+            if (SPLIT)
+                put_split(snext, plane, off, sO32[0 * TS * LDO + a * LDO + b], -sO32[1 * TS * LDO + a * LDO + b]);
             if (STAGE <= 3) {
                 dnext[off] = sO32[0 * TS * LDO + a * LDO + b];
                 dnext[plane + off] = -sO32[1 * TS * LDO + a * LDO + b];
@@ -561,16 +586,6 @@ __device__ __forceinline__ void mixed_sparse_tile(const DevOps &ops, const Mixed
     __syncthreads();
 }
 
-
-// The gain kernel of the dense (tensor-core) stage: stage 2 also takes the
-// stop decision (CTA blk 0).
-template <int STAGE>
-__device__ __forceinline__ void gain_mixed_body(const DevOps &ops, const MixedWork &w, const float *__restrict__ din,
-                                                int blk, int nblk) {
-    if (STAGE == 2) stage2_decide(w, blk == 0);
-    const int wpb = blockDim.x >> 5;
-    gain_rows(ops, din, blk * wpb, nblk * wpb, ops.np, 0, w.g);
-}
 
 // Refresh, part 1 (one CTA): sigma = 1 / Re tr(y) for y = R + delta, in
 // FP64, and the FP32 forms of dt that the delta stages use.

@@ -44,7 +44,6 @@ struct qpr_ctx {
     float *d_g32 = nullptr, *d_hval32 = nullptr, *d_c32 = nullptr, *d_sval32 = nullptr, *d_partials32 = nullptr;
     __nv_bfloat16 *d_hsplit = nullptr;  // dense mixed form: H split into 3 BF16 planes
     __nv_bfloat16 *d_dsplit = nullptr;  // dense mixed form: 3 delta-split buffers of 6 planes
-    int2 *d_pairs_tc = nullptr;
     qpr::TcMaps tcmaps{};
     void *d_digits = nullptr;   // FP64 dense form on the tensor cores: digit planes, exponents, X
     int *d_digint = nullptr;
@@ -779,7 +778,6 @@ void qpr_destroy(qpr_ctx *ctx) {
     cudaFree(ctx->d_c32);
     cudaFree(ctx->d_hsplit);
     cudaFree(ctx->d_dsplit);
-    cudaFree(ctx->d_pairs_tc);
     cudaFree(ctx->d_g);
     cudaFree(ctx->d_partials);
     cudaFree(ctx->d_pairs);
@@ -987,7 +985,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         CREATE_CUDA(cudaMalloc(&ctx->d_c32, np * sizeof(float)));
         CREATE_CUDA(cudaMemcpy(ctx->d_c32, c32.data(), np * sizeof(float), cudaMemcpyHostToDevice));
     }
-    int npairs_tc = 0;
+    int tc_levels = 1;
     if (tc) {
         CREATE_CUDA(qpr::init_mixed_tc());
         // H = H0 + H1 + H2, each the BF16 rounding of what the previous left
@@ -1004,19 +1002,14 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
                 hs[o2] = h0;
                 hs[plane + o2] = h1;
                 hs[2 * plane + o2] = h2;
+                tc_levels = std::max(tc_levels, __bfloat162float(h2) != 0.0f ? 3 : (__bfloat162float(h1) != 0.0f ? 2 : 1));
             }
         CREATE_CUDA(cudaMalloc(&ctx->d_hsplit, 3 * plane * sizeof(__nv_bfloat16)));
         CREATE_CUDA(cudaMemcpy(ctx->d_hsplit, hs.data(), 3 * plane * sizeof(__nv_bfloat16), cudaMemcpyHostToDevice));
         CREATE_CUDA(cudaMalloc(&ctx->d_dsplit, 18 * plane * sizeof(__nv_bfloat16)));
         CREATE_CUDA(cudaMemset(ctx->d_dsplit, 0, 18 * plane * sizeof(__nv_bfloat16)));
-        const int Ttc = np / qpr::kTileTc;
-        std::vector<int2> ptc;
-        for (int I = 0; I < Ttc; ++I)
-            for (int J = I + 1; J < Ttc; ++J) ptc.push_back(make_int2(I, J));
-        for (int I = 0; I < Ttc; ++I) ptc.push_back(make_int2(I, I));
-        npairs_tc = (int)ptc.size();
-        CREATE_CUDA(cudaMalloc(&ctx->d_pairs_tc, ptc.size() * sizeof(int2)));
-        CREATE_CUDA(cudaMemcpy(ctx->d_pairs_tc, ptc.data(), ptc.size() * sizeof(int2), cudaMemcpyHostToDevice));
+        CREATE_CUDA(cudaMalloc(&ctx->d_X, 2 * plane * sizeof(float)));
+        CREATE_CUDA(cudaMemset(ctx->d_X, 0, 2 * plane * sizeof(float)));
     }
     if (o.precision == QPR_MIXED) {
         CREATE_CUDA(cudaMalloc(&ctx->d_mix64, 4 * plane * sizeof(double)));
@@ -1025,7 +1018,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         CREATE_CUDA(cudaMemset(ctx->d_mix32, 0, 14 * plane * sizeof(float)));
         CREATE_CUDA(cudaMalloc(&ctx->d_g32, 2 * np * sizeof(float)));  // g, then the diagonal vector pv
         CREATE_CUDA(cudaMemset(ctx->d_g32, 0, 2 * np * sizeof(float)));
-        CREATE_CUDA(cudaMalloc(&ctx->d_partials32, std::max<size_t>(pairs.size(), (size_t)npairs_tc) * sizeof(float)));
+        CREATE_CUDA(cudaMalloc(&ctx->d_partials32, pairs.size() * sizeof(float)));
         std::vector<float> sv32(std::max<size_t>(1, sval.size()));
         for (size_t q = 0; q < sval.size(); ++q) sv32[q] = (float)sval[q];
         CREATE_CUDA(cudaMalloc(&ctx->d_sval32, sv32.size() * sizeof(float)));
@@ -1224,14 +1217,14 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         mw.ctl = ctx->d_ctl;
         mw.nstage_partials = (int)pairs.size();
         if (tc) {
-            mw.pairs_tc = ctx->d_pairs_tc;
-            mw.npairs_tc = npairs_tc;
-            mw.nstage_partials = npairs_tc;
+            mw.X = ctx->d_X;
             mw.splitD = ctx->d_dsplit;
             mw.splitA = ctx->d_dsplit + 6 * plane;
             mw.splitB = ctx->d_dsplit + 12 * plane;
             const __nv_bfloat16 *ds[3] = {mw.splitD, mw.splitA, mw.splitB};
-            if (!qpr::make_tc_maps(ops, ctx->d_hsplit, ds, &ctx->tcmaps)) {
+            int sms = 0;
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+            if (!qpr::make_tc_maps(ops, ctx->d_hsplit, tc_levels, sms, ds, &ctx->tcmaps)) {
                 ctx->err = "cuTensorMapEncodeTiled failed";
                 g_create_error = ctx->err;
                 qpr_destroy(ctx);
@@ -1450,7 +1443,7 @@ qpr_status qpr_profile_step(qpr_ctx *ctx, const void *rho, double dt, int64_t st
     h->resid_exact_step = -1;
     QPR_CUDA(ctx, cudaMemcpyAsync(ctx->d_ctl, h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream));
     const bool mixed = ctx->opt.precision == QPR_MIXED;
-    const bool cols = mixed && ctx->mw.cmaps;
+    const bool cols = mixed && (ctx->mw.cmaps || ctx->mw.splitD);
     // every kernel alone on the stream, between two events: kind 0 product,
     // 1 epilogue, 2 gain; the refresh's kernels together (kind 3)
     struct Mark { int kind; cudaEvent_t a, b; };
@@ -1486,12 +1479,7 @@ qpr_status qpr_profile_step(qpr_ctx *ctx, const void *rho, double dt, int64_t st
                     st = timed(1, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 2, true); });
                 if (k == 0) per_step += 2;
             } else if (mixed) {
-                if (ctx->mw.splitD) {
-                    st = timed(2, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 1, true); });
-                    if (k == 0) per_step += 1;
-                }
-                if (st == QPR_OK)
-                    st = timed(0, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 2, true); });
+                st = timed(0, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 2, true); });
                 if (k == 0) per_step += 1;
             } else {
                 st = timed(2, [&] { qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream); });

@@ -175,15 +175,13 @@ struct MixedWork {
     int tiles;
     Ctl *ctl;
     int nstage_partials;  // residual partials the stage-1 kernel writes
-    // dense backend (tcgen05): 128 x 128 tile pairs and the BF16 split planes
-    // [3 levels][2 planes: Re, -Im][np][np] of the stage-1, stage-2 and
-    // stage-3 inputs (D, da, db); null for the sparse backend
-    int2 *pairs_tc;
-    int npairs_tc;
+    // dense backend (tcgen05): the BF16 split planes [3 levels][2 planes: Re,
+    // -Im][np][np] of the stage-1, stage-2 and stage-3 inputs (D, da, db);
+    // null for the sparse backend
     __nv_bfloat16 *splitD, *splitA, *splitB;
     const TcMaps *maps;   // host pointer, used only by the launch code
-    // column-block form of the sparse backend: X = H delta (2 planes) and the
-    // TMA maps of the stage inputs D, da, db (host pointer; null: tile-pair
+    // column-block form of the sparse backend and dense backend: X = H delta
+    // (2 planes); column-block form: the TMA maps of the stage inputs D, da, db (host pointer; null: tile-pair
     // kernel)
     float *X;
     const struct ColMaps *cmaps;
@@ -209,6 +207,8 @@ constexpr int kTileTc = 128;
 struct TcMaps {
     CUtensorMap h;
     CUtensorMap d[3];
+    int levels;  // leading planes of H that are not zero
+    int sms;
 };
 
 constexpr int kTileFp64 = 32;
@@ -285,10 +285,9 @@ cudaError_t launch_small_rk4(const DevOps &ops, const Work &w, int nnz, int limi
 // Reference refresh: R = y = y / tr(y), F = f(R) exactly (FP64), D = 0, exact
 // residual and stop decision.
 void launch_mixed_refresh(const DevOps &ops, const MixedWork &w, cudaStream_t s);
-// One RK4 stage: parts & 1 launches the gain of the stage delta (the
-// tensor-core form; the tile-pair stage kernel forms the gain itself), parts
-// & 2 the stage kernel (3 = both, in that order). Column-block form: parts &
-// 1 the SpMM (its leading CTAs form the gain), parts & 2 the epilogue;
+// One RK4 stage. Column-block and dense forms: parts & 1 launches the product
+// (its leading CTAs form the gain), parts & 2 the epilogue (3 = both, in that
+// order); tile-pair form: parts & 2 the stage kernel, which does everything.
 // serial (profiling): no programmatic dependent launch.
 void launch_mixed_stage(int stage, const DevOps &ops, const MixedWork &w, cudaStream_t s, int parts = 3,
                         bool serial = false);
@@ -296,9 +295,12 @@ void launch_mixed_stage(int stage, const DevOps &ops, const MixedWork &w, cudaSt
 cudaError_t init_stage_mixed();
 // Dense backend of the mixed form (stage_mixed_tc.cu).
 cudaError_t init_mixed_tc();
-bool make_tc_maps(const DevOps &ops, const __nv_bfloat16 *hsplit, const __nv_bfloat16 *const dsplit[3],
-                  TcMaps *maps);
-void launch_mixed_tc(int stage, const DevOps &ops, const MixedWork &w, const TcMaps &m, cudaStream_t s);
+bool make_tc_maps(const DevOps &ops, const __nv_bfloat16 *hsplit, int levels, int sms,
+                  const __nv_bfloat16 *const dsplit[3], TcMaps *maps);
+// X = H delta (with the gain and, at stage 2, the stop decision in its leading CTAs).
+void launch_mixed_tc_product(int stage, const DevOps &ops, const MixedWork &w, const TcMaps &m, cudaStream_t s, bool pdl);
+// The epilogue of the forms that write X (the column forms and the dense one).
+void launch_x_epilogue(int stage, const DevOps &ops, const MixedWork &w, cudaStream_t s, bool pdl);
 // Column-block form of the sparse mixed stage (stage_cols.cu): per stage a
 // column-block SpMM X = H delta from TMA-staged columns, then the tile-pair
 // epilogue. Used where its staged operands fit (np <= kColMaxNp and a plan).

@@ -67,8 +67,10 @@ static_assert(kANT == kENT, "the stop decision sums the residual partials with t
 // stage input, F32, D, S, ...: written two kernels back, complete once the
 // SpMM kernel has passed its own dependency wait) are loaded before
 // grid_dependency_wait; X, the gain and the stop flag after it, together.
-template <int STAGE>
-__global__ void __launch_bounds__(kENT, 3) cols_epi_kernel(DevOps ops, MixedWork w) {
+// SPLIT: the dense form's epilogue (after its product kernel, which likewise
+// waits before it lets this kernel start).
+template <int STAGE, bool SPLIT>
+__global__ void __launch_bounds__(kENT, SPLIT ? 2 : 3) cols_epi_kernel(DevOps ops, MixedWork w) {
     __shared__ __align__(16) float sX1[TS * LDX];
     __shared__ __align__(16) float sX2[TS * LDX];
     __shared__ __align__(16) float sO[4 * TS * LDO];
@@ -88,7 +90,7 @@ __global__ void __launch_bounds__(kENT, 3) cols_epi_kernel(DevOps ops, MixedWork
     __syncthreads();
     if (!s_done) {
         // no ticket: the stage-2 SpMM grid takes the stop decision (gain_role)
-        epilogue_pair_staged<STAGE, false>(ops, w, pr.x, pr.y, pr.z, blockIdx.x == 0, w.npairs, sX1, sX2, sg, sO,
+        epilogue_pair_staged<STAGE, false, SPLIT>(ops, w, pr.x, pr.y, pr.z, blockIdx.x == 0, w.npairs, sX1, sX2, sg, sO,
                                            in);
     }
     timeline::leave();
@@ -410,15 +412,23 @@ void launch_cols_stage(int stage, const DevOps &ops, const MixedWork &w, cudaStr
             }
         }
     }
-    if (parts & 2) {
-        const dim3 ge(w.npairs);
-        switch (stage) {
-            case 1: launch_pdl(cols_epi_kernel<1>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
-            case 2: launch_pdl(cols_epi_kernel<2>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
-            case 3: launch_pdl(cols_epi_kernel<3>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
-            default: launch_pdl(cols_epi_kernel<4>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
-        }
+    if (parts & 2) launch_x_epilogue(stage, ops, w, s, pdl);
+}
+
+template <bool SPLIT>
+void launch_epi(int stage, const DevOps &ops, const MixedWork &w, cudaStream_t s, bool pdl) {
+    const dim3 ge(w.npairs);
+    switch (stage) {
+        case 1: launch_pdl(cols_epi_kernel<1, SPLIT>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
+        case 2: launch_pdl(cols_epi_kernel<2, SPLIT>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
+        case 3: launch_pdl(cols_epi_kernel<3, SPLIT>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
+        default: launch_pdl(cols_epi_kernel<4, SPLIT>, ge, dim3(kENT), 0, s, pdl, ops, w); break;
     }
+}
+
+void launch_x_epilogue(int stage, const DevOps &ops, const MixedWork &w, cudaStream_t s, bool pdl) {
+    if (w.splitD) launch_epi<true>(stage, ops, w, s, pdl);
+    else launch_epi<false>(stage, ops, w, s, pdl);
 }
 
 cudaError_t raise_smem_limit(const void *kernel, int bytes) {

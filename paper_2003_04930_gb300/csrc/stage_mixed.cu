@@ -50,16 +50,6 @@ cudaError_t set_mixed_attr() {
                                 kMixedDynSmem);
 }
 
-template <int STAGE>
-__global__ void __launch_bounds__(256)
-gain_mixed_kernel(DevOps ops, MixedWork w, const float *__restrict__ din) {
-    __shared__ int s_done;
-    if (threadIdx.x == 0) s_done = *(volatile int *)&w.ctl->done;
-    __syncthreads();
-    if (s_done) return;
-    gain_mixed_body<STAGE>(ops, w, din, blockIdx.x, gridDim.x);
-}
-
 __global__ void __launch_bounds__(256) refresh_trace_kernel(DevOps ops, MixedWork w) {
     __shared__ int s_done;
     if (threadIdx.x == 0) s_done = *(volatile int *)&w.ctl->done;
@@ -124,22 +114,12 @@ void launch_mixed_stage(int stage, const DevOps &ops, const MixedWork &w, cudaSt
         launch_cols_stage(stage, ops, w, s, parts, serial);
         return;
     }
-    const float *din = (stage == 1) ? w.D : (stage == 3 ? w.db : w.da);
-    int gb = (ops.np + 7) / 8;
-    if (gb > 152) gb = 152;
-    // the sparse stage kernel computes the gain and the stop decision itself
-    if ((parts & 1) && w.splitD) {
-        switch (stage) {
-            case 1: gain_mixed_kernel<1><<<gb, 256, 0, s>>>(ops, w, din); break;
-            case 2: gain_mixed_kernel<2><<<gb, 256, 0, s>>>(ops, w, din); break;
-            case 3: gain_mixed_kernel<3><<<gb, 256, 0, s>>>(ops, w, din); break;
-            default: gain_mixed_kernel<4><<<gb, 256, 0, s>>>(ops, w, din); break;
-        }
-    }
-    if ((parts & 2) && w.splitD) {
-        launch_mixed_tc(stage, ops, w, *w.maps, s);
+    if (w.splitD) {  // dense form: the same two launches
+        if (parts & 1) launch_mixed_tc_product(stage, ops, w, *w.maps, s, !serial);
+        if (parts & 2) launch_x_epilogue(stage, ops, w, s, !serial);
         return;
     }
+    // the sparse stage kernel computes the gain and the stop decision itself
     if (parts & 2) {
         switch (stage) {
             case 1: stage_mixed_sparse_kernel<1><<<w.npairs, NT, kMixedDynSmem, s>>>(ops, w); break;
