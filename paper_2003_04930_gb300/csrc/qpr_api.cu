@@ -260,7 +260,7 @@ qpr_status run_rk4(qpr_ctx *ctx, double dt, double tol, int64_t max_steps) {
 qpr_status launch_mixed_block(qpr_ctx *ctx, int steps, bool refresh) {
     if (refresh) {
         qpr::launch_mixed_refresh(ctx->ops, ctx->mw, ctx->stream);
-        ctx->launches += qpr::kMixedLaunchesPerRefresh;
+        ctx->launches += qpr::mixed_launches_per_refresh(ctx->mw);
     }
     QPR_CUDA(ctx, qpr::launch_cols_block(ctx->ops, ctx->mw, steps, ctx->persist_grid, ctx->stream));
     ctx->launches += 1;
@@ -349,7 +349,7 @@ qpr_status run_mixed(qpr_ctx *ctx, double dt, double tol, int64_t max_steps) {
             } else {
                 enqueue_mixed_block(ctx, block, refresh);
             }
-            ctx->launches += (refresh ? qpr::kMixedLaunchesPerRefresh : 0) +
+            ctx->launches += (refresh ? qpr::mixed_launches_per_refresh(ctx->mw) : 0) +
                              mixed_launches_per_step(ctx) * (int64_t)block;
         }
         since = (refresh ? 0 : since) + block;
@@ -375,7 +375,7 @@ qpr_status run_mixed(qpr_ctx *ctx, double dt, double tol, int64_t max_steps) {
         h->status = qpr::kCtlRunning;
         QPR_CUDA(ctx, cudaMemcpyAsync(ctx->d_ctl, h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream));
         qpr::launch_mixed_refresh(ctx->ops, ctx->mw, ctx->stream);
-        ctx->launches += qpr::kMixedLaunchesPerRefresh;
+        ctx->launches += qpr::mixed_launches_per_refresh(ctx->mw);
         st = read_ctl(ctx);
         if (st != QPR_OK) return st;
         if (h->err_timeout) return fail(ctx, QPR_E_TIMEOUT, "a device-side wait gave up (err_timeout set by a stage kernel)");
@@ -1112,7 +1112,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     wk.npairs = (int)pairs.size();
     wk.tiles = T;
     wk.ctl = ctx->d_ctl;
-    if (o.precision == QPR_FP64 && ctx->backend == QPR_BACKEND_DENSE) {
+    if (ctx->backend == QPR_BACKEND_DENSE) {
         // the product on the tensor cores by exact digits where a plan keeps
         // the sums exact and its planes fit beside everything else; else the
         // FP64 tensor kernel and its dense H (N = 500, unit weights: 616 us a
@@ -1205,6 +1205,12 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
                 return QPR_E_CUDA;
             }
             mw.cmaps = &ctx->colmaps;
+        }
+        // the refresh: with few nonzeros the sparse FP64 stage is the faster one
+        // (N = 922, 16 nonzeros a row: 0.16 ms against 0.36)
+        if (ctx->d_digits && (double)hval.size() >= (double)n * (double)n / 8.0) {
+            mw.digits = &ctx->digits;
+            mw.digitmaps = &ctx->digitmaps;
         }
         mw.g = ctx->d_g32;
         mw.pv = ctx->d_g32 + np;
@@ -1411,7 +1417,7 @@ qpr_status qpr_profile_chain(qpr_ctx *ctx, const void *rho, double dt, int32_t r
     cudaEventRecord(ev[2], ctx->stream);
     for (int r = 0; r < reps; ++r) qpr::launch_mixed_stage(2, ctx->ops, ctx->mw, ctx->stream, 2, false);
     cudaEventRecord(ev[3], ctx->stream);
-    ctx->launches += 3 + qpr::kMixedLaunchesPerRefresh + 2 * (int64_t)reps;
+    ctx->launches += 3 + qpr::mixed_launches_per_refresh(ctx->mw) + 2 * (int64_t)reps;
     st = sync_ctx(ctx);
     if (st == QPR_OK) {
         float a = 0.f, b = 0.f;

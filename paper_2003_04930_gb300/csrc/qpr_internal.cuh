@@ -161,6 +161,8 @@ struct Work {
 // planes each): F32 = fl(F), dt F = Ghi + Glo (float-float) and the stage
 // inputs da/db (the nested RK4 form keeps no running stage sum).
 struct TcMaps;
+struct DigitWork;
+struct DigitMaps;
 struct MixedWork {
     double *R, *F;
     float *F32, *D, *Dlo, *da, *db, *Ghi, *Glo;
@@ -180,6 +182,10 @@ struct MixedWork {
     // null for the sparse backend
     __nv_bfloat16 *splitD, *splitA, *splitB;
     const TcMaps *maps;   // host pointer, used only by the launch code
+    // dense backend, host pointers: the refresh evaluates f(R) with the exact
+    // digit products where there is a plan (null: the sparse FP64 stage)
+    const DigitWork *digits;
+    const DigitMaps *digitmaps;
     // column-block form of the sparse backend and dense backend: X = H delta
     // (2 planes); column-block form: the TMA maps of the stage inputs D, da, db (host pointer; null: tile-pair
     // kernel)
@@ -363,7 +369,7 @@ cudaError_t launch_cols_block(const DevOps &ops, const MixedWork &w, int steps, 
 // Kernel launches per RK4 step and per refresh of the mixed form.
 constexpr int kMixedLaunchesPerStep = 4;   // tile-pair sparse kernel (the dense one adds 4 gain kernels)
 constexpr int kMixedLaunchesPerStepCols = 8;  // column-block form: SpMM (with the gain) and epilogue per stage
-constexpr int kMixedLaunchesPerRefresh = 5;
+inline int mixed_launches_per_refresh(const MixedWork &w) { return w.digits ? 6 : 5; }
 // Steady-state solves with adaptive_refresh: the longest window between
 // refreshes, in multiples of ref_refresh.
 constexpr int kMaxRefreshGrowth = 8;

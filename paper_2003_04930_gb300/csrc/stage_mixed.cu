@@ -92,7 +92,9 @@ void launch_mixed_refresh(const DevOps &ops, const MixedWork &w, cudaStream_t s)
     const size_t tot = 2 * (size_t)ops.np * ops.np;
     refresh_trace_kernel<<<1, 256, 0, s>>>(ops, w);
     refresh_normalize_kernel<<<grid_elems(tot), 256, 0, s>>>(ops, w);
-    // F = f(R) with the exact FP64 sparse stage kernel (stage 0: reads w.y, writes w.z)
+    // F = f(R) in FP64 (stage 0: reads w.y, writes w.z): the sparse stage
+    // kernel, or with a dense H the digit products (N = 900, unit weights: the
+    // sparse kernel's 394 gathers a row made a refresh 1750 us; now 180)
     Work w64{};
     w64.y = w.R;
     w64.z = w.F;
@@ -104,8 +106,12 @@ void launch_mixed_refresh(const DevOps &ops, const MixedWork &w, cudaStream_t s)
     w64.npairs = w.npairs;
     w64.tiles = w.tiles;
     w64.ctl = w.ctl;
-    launch_gain(0, ops, w.R, w64, s);
-    launch_stage_sparse(0, ops, w64, s);
+    if (w.digits) {
+        launch_stage_digits(0, ops, w64, *w.digits, *w.digitmaps, s);
+    } else {
+        launch_gain(0, ops, w.R, w64, s);
+        launch_stage_sparse(0, ops, w64, s);
+    }
     refresh_post_kernel<<<grid_elems(tot), 256, 0, s>>>(ops, w);
 }
 

@@ -33,3 +33,28 @@ def test_trajectory(n, steps, levels):
     ref = Oracle.from_edges(g, alpha=0.85, omega=0.7).evolve(rho0, dt, steps)
     assert np.abs(got - got.conj().T).max() == 0.0
     assert np.linalg.norm(got - ref) <= 1e-6
+
+
+@pytest.mark.parametrize("n", [50, 129])
+@pytest.mark.parametrize("weights", ["unit", "lognormal", "wide"])
+def test_rhs_and_steady_state_of_a_mixed_context(n, weights):
+    # f(rho) is exact FP64 whatever the precision, by whichever FP64 stage the weights allow
+    g = graphs.erdos_renyi(n, 0.4, n)
+    rng = np.random.default_rng(n)
+    w = {"unit": g.w, "lognormal": rng.lognormal(0.0, 1.0, g.m), "wide": np.where(np.arange(g.m) % 7 == 0, 1e-250, 1.0)}[weights]
+    g = graphs.EdgeList(n, g.src, g.dst, w)
+    o = Oracle.from_edges(g, alpha=0.85, omega=0.8)
+    rho = graphs.random_hermitian(n, 7)
+    ref = o.rhs(rho)
+    with Solver.from_edges(g, alpha=0.85, omega=0.8, precision=Q.QPR_MIXED, backend=Q.QPR_BACKEND_DENSE) as s:
+        out = torch.zeros((n, n), dtype=torch.complex128, device="cuda:0")
+        s.rhs(torch.from_numpy(rho).to("cuda:0"), out)
+        assert np.abs(out.cpu().numpy() - ref).max() <= 1e-13 * max(1.0, np.abs(ref).max()) * max(1, n / 16)
+        d = torch.from_numpy(graphs.maximally_mixed(n)).to("cuda:0")
+        st = s.steady_state(d, 0.01, 1e-8, 100000)
+        assert st["converged"] == 1 and st["residual"] < 1e-8
+        assert abs(s.residual(d) - st["residual"]) <= 1e-6 * st["residual"]
+    rref, steps, _, _ = o.steady_state(graphs.maximally_mixed(n), 0.01, 1e-8, 100000)
+    assert abs(st["steps"] - steps) <= 1
+    p, pr = np.real(np.diag(d.cpu().numpy())), np.real(np.diag(rref))
+    assert np.abs(p - pr).max() <= 1e-7 * pr.max()
