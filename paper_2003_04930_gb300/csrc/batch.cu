@@ -96,14 +96,6 @@ __global__ void __launch_bounds__(256) b_normalize_kernel(const BatchGraph *gs, 
                                   (size_t)gridDim.x * blockDim.x);
 }
 
-__global__ void __launch_bounds__(256) b_gain64_kernel(const BatchGraph *gs, const int *act, const uint8_t *due) {
-    __shared__ BatchGraph sg;
-    __shared__ int s_flag;
-    load_graph(gs, act[blockIdx.x], sg);
-    if (skip_refresh(sg, act[blockIdx.x], due, &s_flag)) return;
-    gain64::gain_fp64_body(0, sg.ops, sg.w64, sg.w64.y, (size_t)sg.ops.np + 1, 0, 1);
-}
-
 __global__ void __launch_bounds__(sparse64::NTHREADS)
 b_sparse64_kernel(const BatchGraph *gs, const int4 *items, int nitems, const uint8_t *due) {
     extern __shared__ __align__(16) double smem[];
@@ -292,7 +284,6 @@ void launch_refresh(const BatchGraph *gs, const Lists &L, int max_np, cudaStream
     const dim3 eg(elem_chunks(max_np), L.nact);
     b_trace_kernel<<<L.nact, 256, 0, s>>>(gs, L.act, due);
     b_normalize_kernel<<<eg, 256, 0, s>>>(gs, L.act, due);
-    b_gain64_kernel<<<L.nact, 256, 0, s>>>(gs, L.act, due);
     b_sparse64_kernel<<<std::min(L.nitems, 152 * 3), sparse64::NTHREADS, sparse64::SMEM_BYTES, s>>>(gs, L.items,
                                                                                                      L.nitems, due);
     b_post_kernel<<<eg, 256, 0, s>>>(gs, L.act, due);

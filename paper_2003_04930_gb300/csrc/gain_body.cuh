@@ -42,52 +42,49 @@ __device__ __forceinline__ double block_sum(double v, double *red, G grp = G{}) 
     return s;
 }
 
+// The stop decision of stage 2: the residual partials of stage 1 summed in
+// index order into ||f(y_n)||_F of the normalised state. One group of threads.
+template <typename G = Cta>
+__device__ __forceinline__ void stop_decision(const Work &w, double *red, G grp = G{}) {
+    Ctl *ctl = w.ctl;
+    double s = 0.0;
+    for (int i = grp.tid(); i < w.npairs; i += grp.size()) s += w.partials[i];
+    s = block_sum(s, red, grp);
+    if (grp.tid() == 0) {
+        const double r = ctl->scale * sqrt(s);
+        ctl->resid = r;
+        ctl->resid_step = ctl->step;
+        if (!isfinite(r)) {
+            ctl->status = kCtlNonFinite;
+            ctl->done = 1;
+        } else if (r < ctl->tol) {
+            ctl->status = kCtlConverged;
+            ctl->done = 1;
+        } else if (ctl->step >= ctl->max_steps) {
+            ctl->status = kCtlMaxSteps;
+            ctl->done = 1;
+        }
+    }
+}
+
+// out[i - base] = g_i for rows i = r0 + (warp of the group), + step, ... < r1,
 // g = G p with G = alpha S + (1 - alpha) F (Eq. S2, Eq. S4), p_j = Y_jj
 // (diag[j stride]):
 //   (S p)_i = sum_{j with out-links} A_ij / outDeg(j) p_j  +  dangling part,
 //   dangling part = (D - [i dangles] p_i) / (N - 1)  (F columns)  or  D / N,
 //   (F p)_i = (P - p_i) / (N - 1),
-// with P = sum_j p_j and D = sum over dangling j of p_j.
-// Stage 1 also publishes 1 / Re tr(y), by which stage 4 normalises the step.
-// Stage 2 first reduces the residual partials of stage 1 into ||f(y_n)||_F of
-// the normalised state and takes the stop decision (one CTA).
-// blk / nblk: this group's index and the number of groups sharing the rows; the
-// residual decision (stage 2) is taken by blk 0.
+// with P = sum_j p_j and D = sum over dangling j of p_j. With `publish` (one
+// group of stage 1) it also sets 1 / Re tr(y), by which stage 4 normalises.
 template <typename G = Cta>
-__device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, const Work &w,
-                                               const double *__restrict__ diag, size_t stride, int blk, int nblk,
-                                               G grp = G{}) {
-    __shared__ double red[32];
-    Ctl *ctl = w.ctl;
-    const int n = ops.n, np = ops.np;
-
-    if (stage == 2 && blk == 0) {
-        double s = 0.0;
-        for (int i = grp.tid(); i < w.npairs; i += grp.size()) s += w.partials[i];
-        s = block_sum(s, red, grp);
-        if (grp.tid() == 0) {
-            const double r = ctl->scale * sqrt(s);
-            ctl->resid = r;
-            ctl->resid_step = ctl->step;
-            if (!isfinite(r)) {
-                ctl->status = kCtlNonFinite;
-                ctl->done = 1;
-            } else if (r < ctl->tol) {
-                ctl->status = kCtlConverged;
-                ctl->done = 1;
-            } else if (ctl->step >= ctl->max_steps) {
-                ctl->status = kCtlMaxSteps;
-                ctl->done = 1;
-            }
-        }
-    }
-
+__device__ __forceinline__ void gain_rows(const DevOps &ops, Ctl *ctl, const double *__restrict__ diag, size_t stride,
+                                          int r0, int step, int r1, int base, double *out, bool publish, double *red,
+                                          G grp = G{}) {
+    const int n = ops.n;
     // independent of the sums below: the reciprocal, and the row sum of this
     // warp's first row, whose loads then fly with those of the diagonal
     const double inv_nm1 = __drcp_rn((double)(n - 1));
     const int lane = threadIdx.x & 31;
-    const int wpb = grp.size() >> 5;
-    const int first = blk * wpb + (grp.tid() >> 5);
+    const int first = r0 + (grp.tid() >> 5);
     auto row_part = [&](int i) {
         double s = 0.0;
         if (i < n) {
@@ -96,7 +93,7 @@ __device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, con
         }
         return s;
     };
-    double s0 = row_part(first);
+    const double s0 = first < r1 ? row_part(first) : 0.0;
     double P = 0.0, D = 0.0;
     for (int j = grp.tid(); j < n; j += grp.size()) {
         const double pj = diag[j * stride];
@@ -105,7 +102,7 @@ __device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, con
     }
     P = block_sum(P, red, grp);
     D = block_sum(D, red, grp);
-    if (stage == 1 && blk == 0 && grp.tid() == 0) {
+    if (publish && grp.tid() == 0) {
         ctl->scale = 1.0 / P;
         ctl->trace = P;
         if (!(P > 0.0) || !isfinite(P)) {
@@ -113,7 +110,7 @@ __device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, con
             ctl->done = 1;
         }
     }
-    for (int i = first; i < np; i += nblk * wpb) {
+    for (int i = first; i < r1; i += step) {
         const double s = warp_sum(i == first ? s0 : row_part(i));
         if (lane == 0) {
             double gi = 0.0;
@@ -125,9 +122,21 @@ __device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, con
                 gi = __fma_rn(ops.alpha, __dadd_rn(s, dterm),
                               __dmul_rn(__dmul_rn(__dsub_rn(1.0, ops.alpha), __dsub_rn(P, pi)), inv_nm1));
             }
-            w.g[i] = gi;
+            out[i - base] = gi;
         }
     }
+}
+
+// The gain of a stage into w.g by nblk groups of threads, this one blk; stage
+// 1 publishes the scale, stage 2 takes the stop decision (group 0 both).
+template <typename G = Cta>
+__device__ __forceinline__ void gain_fp64_body(int stage, const DevOps &ops, const Work &w,
+                                               const double *__restrict__ diag, size_t stride, int blk, int nblk,
+                                               G grp = G{}) {
+    __shared__ double red[32];
+    if (stage == 2 && blk == 0) stop_decision(w, red, grp);
+    const int wpb = grp.size() >> 5;
+    gain_rows(ops, w.ctl, diag, stride, blk * wpb, nblk * wpb, ops.np, 0, w.g, stage == 1 && blk == 0, red, grp);
 }
 
 }  // namespace gain64

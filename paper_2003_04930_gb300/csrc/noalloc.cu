@@ -36,11 +36,11 @@ constexpr size_t kOffZ = 2 * kPlane;              // 2 planes: f(rho)
 constexpr size_t kOffG = 4 * kPlane;              // gain, kMaxNp
 constexpr size_t kOffC = kOffG + kMaxNp;          // column sums of G, kMaxNp
 constexpr size_t kOffPart = kOffC + kMaxNp;       // residual partials, kMaxPairs
-constexpr size_t kOffPairs = kOffPart + kMaxPairs;  // int2 table, one double each
-constexpr size_t kOffCtl = kOffPairs + kMaxPairs;
+constexpr size_t kOffPairs = kOffPart + kMaxPairs;  // int4 table, two doubles each
+constexpr size_t kOffCtl = kOffPairs + 2 * kMaxPairs;
 constexpr size_t kCtlDoubles = (sizeof(qpr::Ctl) + sizeof(double) - 1) / sizeof(double);
 constexpr size_t kScratchDoubles = kOffCtl + kCtlDoubles;
-static_assert(sizeof(int2) == sizeof(double), "one pair per double slot");
+static_assert(sizeof(int4) == 2 * sizeof(double) && kOffPairs % 2 == 0, "one pair per two double slots, aligned");
 
 // The scratch array. In host code its name is only a host-side stand-in:
 // the device address comes from cudaGetSymbolAddress (see scratch_base).
@@ -70,8 +70,8 @@ __global__ void noalloc_setup_kernel(qpr::DevOps ops, qpr::Work w, double *c) {
         ctl->resid_step = 0;
         int q = 0;
         for (int I = 0; I < T; ++I)
-            for (int J = I + 1; J < T; ++J) w.pairs[q++] = make_int2(I, J);
-        for (int I = 0; I < T; ++I) w.pairs[q++] = make_int2(I, I);
+            for (int J = I + 1; J < T; ++J, ++q) w.pairs64[q] = make_int4(I, J, q, 0);
+        for (int I = 0; I < T; ++I, ++q) w.pairs64[q] = make_int4(I, I, q, 0);
     }
     const int nnz = ops.s_ptr[n];
     for (int j = threadIdx.x; j < np; j += blockDim.x) {
@@ -158,14 +158,13 @@ extern "C" qpr_status qpr_rhs_noalloc(int64_t n, const int32_t *h_ptr, const int
     w.yb = w.y;
     w.g = base + kOffG;
     w.partials = base + kOffPart;
-    w.pairs = reinterpret_cast<int2 *>(base + kOffPairs);
+    w.pairs64 = reinterpret_cast<int4 *>(base + kOffPairs);
     w.npairs = T * (T + 1) / 2;
     w.tiles = T;
     w.ctl = reinterpret_cast<qpr::Ctl *>(base + kOffCtl);
 
     noalloc_setup_kernel<<<1, 256, 0, s>>>(ops, w, base + kOffC);
     qpr::launch_import((const double *)rho, (int)n, np, w.y, s);
-    qpr::launch_gain(0, ops, w.y, w, s);
     qpr::launch_stage_sparse(0, ops, w, s);
     qpr::launch_export(w.z, (int)n, np, w.ctl, 0, (double *)out, s);
     return cudaGetLastError() == cudaSuccess ? QPR_OK : QPR_E_CUDA;

@@ -61,7 +61,7 @@ struct qpr_ctx {
     double *d_g = nullptr;
     double *d_partials = nullptr;
     int2 *d_pairs = nullptr;
-    int4 *d_epi_pairs = nullptr;
+    int4 *d_epi_pairs = nullptr, *d_pairs64 = nullptr;
     Ctl *d_ctl = nullptr;
     double *d_io = nullptr;     // staging for host density matrices (interleaved)
     double *d_p = nullptr;      // populations staging
@@ -147,12 +147,12 @@ void enqueue_step(qpr_ctx *ctx) {
     const qpr::Work &w = ctx->work;
     const double *yin[5] = {w.y, w.y, w.ya, w.yb, w.ya};
     for (int s = 1; s <= 4; ++s) {
-        if (!ctx->d_digits) qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream);
+        if (ctx->d_H) qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream);
         launch_stage(ctx, s);
     }
 }
 
-int fp64_launches_per_step(const qpr_ctx *ctx) { return 4 * (ctx->d_digits ? qpr::kDigitLaunches : 2); }
+int fp64_launches_per_step(const qpr_ctx *ctx) { return 4 * (ctx->d_digits ? qpr::kDigitLaunches : ctx->d_H ? 2 : 1); }
 
 qpr_status ensure_graph(qpr_ctx *ctx) {
     if (ctx->graph || ctx->opt.graph_steps <= 0) return QPR_OK;
@@ -782,6 +782,7 @@ void qpr_destroy(qpr_ctx *ctx) {
     cudaFree(ctx->d_partials);
     cudaFree(ctx->d_pairs);
     cudaFree(ctx->d_epi_pairs);
+    cudaFree(ctx->d_pairs64);
     cudaFree(ctx->d_ctl);
     cudaFree(ctx->d_io);
     cudaFree(ctx->d_p);
@@ -921,6 +922,11 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     for (int I = 0; I < T; ++I) pairs.push_back(make_int2(I, I));
     CREATE_CUDA(cudaMalloc(&ctx->d_pairs, pairs.size() * sizeof(int2)));
     CREATE_CUDA(cudaMemcpy(ctx->d_pairs, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    {
+        const std::vector<int4> p64 = qpr::pairs_by_work(hops, np);
+        CREATE_CUDA(cudaMalloc(&ctx->d_pairs64, p64.size() * sizeof(int4)));
+        CREATE_CUDA(cudaMemcpy(ctx->d_pairs64, p64.data(), p64.size() * sizeof(int4), cudaMemcpyHostToDevice));
+    }
     {
         // The order of the column-block epilogues' CTAs. Each pair keeps its
         // index in `pairs` (its residual partial slot), so only the schedule
@@ -1109,6 +1115,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     wk.g = ctx->d_g;
     wk.partials = ctx->d_partials;
     wk.pairs = ctx->d_pairs;
+    wk.pairs64 = ctx->d_pairs64;
     wk.npairs = (int)pairs.size();
     wk.tiles = T;
     wk.ctl = ctx->d_ctl;
@@ -1217,6 +1224,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         mw.g64 = ctx->d_g;
         mw.partials = ctx->d_partials;
         mw.pairs = ctx->d_pairs;
+        mw.pairs64 = ctx->d_pairs64;
         mw.epi_pairs = ctx->d_epi_pairs;
         mw.npairs = (int)pairs.size();
         mw.tiles = T;
@@ -1264,7 +1272,7 @@ static qpr_status rhs_impl(qpr_ctx *ctx, const void *rho, void *out, double *res
     memset(h, 0, sizeof(Ctl));
     h->scale = 1.0;
     QPR_CUDA(ctx, cudaMemcpyAsync(ctx->d_ctl, h, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->stream));
-    if (!ctx->d_digits) qpr::launch_gain(0, ctx->ops, ctx->work.y, ctx->work, ctx->stream);
+    if (ctx->d_H) qpr::launch_gain(0, ctx->ops, ctx->work.y, ctx->work, ctx->stream);
     launch_stage(ctx, 0);
     if (out) {
         st = export_rho(ctx, ctx->work.z, 0, out);

@@ -149,6 +149,7 @@ struct Work {
     double *g;            // gain G p of the current stage, np entries
     double *partials;     // one residual partial per stage-kernel CTA
     int2 *pairs;          // tile pairs (I, J), I <= J, off-diagonal first
+    int4 *pairs64;        // the same as {I, J, index in pairs, 0}, most work first (sparse stage)
     int npairs;
     int tiles;            // np / kTileFp64
     Ctl *ctl;
@@ -171,7 +172,8 @@ struct MixedWork {
     double *g64;          // FP64 gain used by the refresh, np
     double *partials;     // exact residual partials of the refresh
     float *partials32;    // residual-estimate partials of the stage-1 kernel
-    int2 *pairs;          // 32 x 32 tile pairs (refresh and sparse stage kernel)
+    int2 *pairs;          // 32 x 32 tile pairs (tile-pair stage kernel)
+    int4 *pairs64;        // the same for the refresh (Work::pairs64)
     int4 *epi_pairs;      // the same pairs in the column-block epilogues' CTA order: {I, J, index in pairs, 0}
     int npairs;
     int tiles;
@@ -272,7 +274,10 @@ void launch_stage_digits(int stage, const DevOps &ops, const Work &w, const Digi
                          cudaStream_t s);
 constexpr int kDigitLaunches = 3;
 
-// ---- sparse (CSR H) FP64 stage kernel (stage_sparse.cu), same contract ----
+// ---- sparse (CSR H) FP64 stage kernel (stage_sparse.cu), same contract; it
+// forms the gain itself ----
+// The tile pairs of an np x np problem, the ones with most nonzeros first.
+std::vector<int4> pairs_by_work(const HostOps &h, int np);
 void launch_stage_sparse(int stage, const DevOps &ops, const Work &w, cudaStream_t s);
 cudaError_t init_stage_sparse();
 
@@ -354,7 +359,7 @@ constexpr int kRkfLaunchesPerAttempt = 2 * kRkfStages;
 bool make_rkf_map(const DevOps &ops, const float *d1, ColMaps *maps);
 void launch_rkf_stage(int stage, const DevOps &ops, const MixedWork &w, cudaStream_t s);
 void launch_rkf_refresh(const DevOps &ops, const MixedWork &w, cudaStream_t s);
-constexpr int kRkfLaunchesPerRefresh = 5;
+constexpr int kRkfLaunchesPerRefresh = 4;
 cudaError_t init_rkf(int spmm_smem, bool gather);
 
 // Persistent form (stage_persist.cu): one cooperative launch runs up to
@@ -369,7 +374,7 @@ cudaError_t launch_cols_block(const DevOps &ops, const MixedWork &w, int steps, 
 // Kernel launches per RK4 step and per refresh of the mixed form.
 constexpr int kMixedLaunchesPerStep = 4;   // tile-pair sparse kernel (the dense one adds 4 gain kernels)
 constexpr int kMixedLaunchesPerStepCols = 8;  // column-block form: SpMM (with the gain) and epilogue per stage
-inline int mixed_launches_per_refresh(const MixedWork &w) { return w.digits ? 6 : 5; }
+inline int mixed_launches_per_refresh(const MixedWork &w) { return w.digits ? 6 : 4; }
 // Steady-state solves with adaptive_refresh: the longest window between
 // refreshes, in multiples of ref_refresh.
 constexpr int kMaxRefreshGrowth = 8;

@@ -405,7 +405,7 @@ constexpr int ET = 256;
 template <int STAGE>
 __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, const double *__restrict__ x) {
     extern __shared__ __align__(16) double sm[];
-    __shared__ double red[ET / 32];
+    __shared__ double red[ET / 32], sg[kEpiTS];
     __shared__ int s_done;
     const int I = w.pairs[blockIdx.x].x, J = w.pairs[blockIdx.x].y;
     const bool diag = I == J;
@@ -428,9 +428,10 @@ __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, cons
             sX2[a * LDX + kEpiTS + lane] = __ldcg(s2 + plane);
         }
     }
+    if (diag && threadIdx.x < kEpiTS) sg[threadIdx.x] = __ldcg(w.g + I * kEpiTS + threadIdx.x);
     __syncthreads();
     if (s_done) return;
-    stage_epilogue<STAGE, ET>(ops, w, I, J, diag, in, sX1, sX2, LDX, red, blockIdx.x, blockIdx.x == 0);
+    stage_epilogue<STAGE, ET>(ops, w, I, J, diag, in, sX1, sX2, LDX, sg, red, blockIdx.x, blockIdx.x == 0);
 }
 
 template <typename K, typename... A>

@@ -165,7 +165,7 @@ stage_fp64_kernel(DevOps ops, Work w) {
             }
     __syncthreads();
     __shared__ double red[NTHREADS / 32];
-    stage_epilogue<STAGE, NTHREADS>(ops, w, I, J, diag, in, sX1, sX2, LDX, red, blockIdx.x, blockIdx.x == 0);
+    stage_epilogue<STAGE, NTHREADS>(ops, w, I, J, diag, in, sX1, sX2, LDX, w.g + I * TS, red, blockIdx.x, blockIdx.x == 0);
 }
 
 template <int STAGE>

@@ -103,13 +103,13 @@ void launch_mixed_refresh(const DevOps &ops, const MixedWork &w, cudaStream_t s)
     w64.g = w.g64;
     w64.partials = w.partials;
     w64.pairs = w.pairs;
+    w64.pairs64 = w.pairs64;
     w64.npairs = w.npairs;
     w64.tiles = w.tiles;
     w64.ctl = w.ctl;
     if (w.digits) {
         launch_stage_digits(0, ops, w64, *w.digits, *w.digitmaps, s);
     } else {
-        launch_gain(0, ops, w.R, w64, s);
         launch_stage_sparse(0, ops, w64, s);
     }
     refresh_post_kernel<<<grid_elems(tot), 256, 0, s>>>(ops, w);
