@@ -44,207 +44,335 @@ constexpr int OFF_BO = OFF_WO + W;
 static_assert(OFF_BO + 1 == kParams, "parameter layout");
 
 // ---------------------------------------------------------------- kernels
-// Y[i][:] (+)= sum_q val[q] X[col[q]][:], d <= 64 columns, one warp per row.
-__global__ void spmm_rows_kernel(const int *__restrict__ ptr, const int *__restrict__ col,
-                                 const float *__restrict__ val, const float *__restrict__ X, float *__restrict__ Y,
-                                 int n, int d, int accumulate) {
+// One graph of a group: its arrays and its part of the workspace, on the
+// device. Every kernel runs over a group of graphs at once (blockIdx.y is the
+// graph): a graph of a few hundred nodes is a few CTAs, and a pass over it is
+// a chain of launches, so a mini-batch of eight takes little longer than one.
+// Each output is still one sum in the order of a pass over the graph alone,
+// and the graphs' gradients are added in the order of the mini-batch.
+struct GnnDev {
+    int n, nblk;                   // nodes, blocks of kRowsWG rows
+    const float *x;                // n x FIN
+    const int *pptr, *pcol, *tptr, *tcol;
+    const float *pval, *tval;      // P and P^T
+    const double *p;               // target populations (or null)
+    float *H, *M, *Z;              // per layer 1..4: n x W each (layer l at (l - 1) n W)
+    float *dA, *dB, *dT;           // n x W: gradients of a layer's output (alternating) and of P h
+    float *s, *ds;                 // n: logits and their gradients
+    double *e, *p_hat;             // n
+    float *part;                   // nblk x kParams: gradient partials
+    double *loss;                  // [0] the graph's loss, [1] log-sum-exp, [2] sum of p
+};
+
+// One row of sum_q val[q] X[col[q]][:], d <= 64 columns (lane and lane + 32),
+// in entry order. 16 entries' loads are in flight at once: with one at a time
+// a hub row of some hundred entries held its launch for 100 us.
+__device__ __forceinline__ void row_sum(const int *__restrict__ col, const float *__restrict__ val, int q0, int q1,
+                                        const float *__restrict__ X, int d, float &a0, float &a1) {
+    constexpr int U = 16;
     const int lane = threadIdx.x & 31;
-    const int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= n) return;
-    float a0 = 0.f, a1 = 0.f;
-    for (int q = ptr[i]; q < ptr[i + 1]; ++q) {
-        const float v = val[q];
-        const float *x = X + (size_t)col[q] * d;
-        if (lane < d) a0 = __fmaf_rn(v, x[lane], a0);
-        if (lane + 32 < d) a1 = __fmaf_rn(v, x[lane + 32], a1);
+    const bool c0 = lane < d, c1 = lane + 32 < d;
+    a0 = a1 = 0.f;
+    for (int qb = q0; qb < q1; qb += 32) {
+        const int m = min(32, q1 - qb);
+        const int k = lane < m ? col[qb + lane] : 0;
+        const float v = lane < m ? val[qb + lane] : 0.f;
+        for (int e = 0; e < m; e += U) {
+            float x0[U], x1[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float *x = X + (size_t)__shfl_sync(0xffffffffu, k, (e + u) & 31) * d + lane;
+                const bool on = e + u < m;
+                x0[u] = on && c0 ? x[0] : 0.f;
+                x1[u] = on && c1 ? x[32] : 0.f;
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const float vu = __shfl_sync(0xffffffffu, v, (e + u) & 31);
+                if (e + u < m) {  // uniform: adding 0 could turn -0 into 0
+                    a0 = __fmaf_rn(vu, x0[u], a0);
+                    a1 = __fmaf_rn(vu, x1[u], a1);
+                }
+            }
+        }
     }
-    float *y = Y + (size_t)i * d;
-    if (lane < d) y[lane] = accumulate ? __fadd_rn(y[lane], a0) : a0;
-    if (lane + 32 < d) y[lane + 32] = accumulate ? __fadd_rn(y[lane + 32], a1) : a1;
 }
 
-// Z = H Ws + M Wn + b, Hout = relu(Z): 32 rows per CTA, 256 threads.
-__global__ void __launch_bounds__(256) dense_fwd_kernel(const float *__restrict__ H, const float *__restrict__ M,
-                                                        const float *__restrict__ prm, int l, int n,
-                                                        float *__restrict__ Z, float *__restrict__ Hout) {
+// Layer l of 8 rows per CTA: M = P h, Z = h Ws + M Wn + b, H = relu(Z); the
+// last layer also forms the logits s = H wo + bo.
+constexpr int kFwdRows = 8;
+__global__ void __launch_bounds__(256) layer_fwd_kernel(const GnnDev *__restrict__ gs, const float *__restrict__ prm,
+                                                        int l) {
     __shared__ float sW[2 * W * W];
-    __shared__ float sH[32 * W], sM[32 * W];
-    const int din = din_of(l);
+    __shared__ float sH[kFwdRows * W], sM[kFwdRows * W], sO[kFwdRows * W];
+    const GnnDev g = gs[blockIdx.y];
+    const int n = g.n, r0 = blockIdx.x * kFwdRows;
+    if (r0 >= n) return;
+    const int din = din_of(l), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t nw = (size_t)n * W;
+    const float *h = l == 1 ? g.x : g.H + (l - 2) * nw;
     for (int t = threadIdx.x; t < 2 * din * W; t += blockDim.x) sW[t] = prm[off_ws(l) + t];  // Ws then Wn
-    const int r0 = blockIdx.x * 32;
-    for (int t = threadIdx.x; t < 32 * din; t += blockDim.x) {
+    for (int t = threadIdx.x; t < kFwdRows * din; t += blockDim.x) {
         const int r = r0 + t / din;
-        sH[t] = r < n ? H[(size_t)r * din + t % din] : 0.f;
-        sM[t] = r < n ? M[(size_t)r * din + t % din] : 0.f;
+        sH[t] = r < n ? h[(size_t)r * din + t % din] : 0.f;
+    }
+    {
+        const int r = r0 + warp;
+        float a0 = 0.f, a1 = 0.f;
+        if (r < n) {
+            row_sum(g.pcol, g.pval, g.pptr[r], g.pptr[r + 1], h, din, a0, a1);
+            float *m = g.M + (l - 1) * nw + (size_t)r * din;
+            if (lane < din) m[lane] = a0;
+            if (lane + 32 < din) m[lane + 32] = a1;
+        }
+        if (lane < din) sM[warp * din + lane] = a0;
+        if (lane + 32 < din) sM[warp * din + lane + 32] = a1;
     }
     __syncthreads();
-    const int f = threadIdx.x & (W - 1);
+    const int f = threadIdx.x & (W - 1), q = threadIdx.x >> 6;  // rows q and q + 4
     const float bf = prm[off_b(l) + f];
-    for (int rr = threadIdx.x >> 6; rr < 32; rr += 4) {
-        const int r = r0 + rr;
-        if (r >= n) break;
-        float z = bf;
-        for (int k = 0; k < din; ++k) {
-            z = __fmaf_rn(sH[rr * din + k], sW[k * W + f], z);
-            z = __fmaf_rn(sM[rr * din + k], sW[din * W + k * W + f], z);
+    float z0 = bf, z1 = bf;
+    for (int k = 0; k < din; ++k) {
+        const float ws = sW[k * W + f], wn = sW[din * W + k * W + f];
+        z0 = __fmaf_rn(sH[q * din + k], ws, z0);
+        z1 = __fmaf_rn(sH[(q + 4) * din + k], ws, z1);
+        z0 = __fmaf_rn(sM[q * din + k], wn, z0);
+        z1 = __fmaf_rn(sM[(q + 4) * din + k], wn, z1);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const int rr = q + 4 * j, r = r0 + rr;
+        const float z = j ? z1 : z0, o = z > 0.f ? z : 0.f;
+        sO[rr * W + f] = o;
+        if (r < n) {
+            g.Z[(l - 1) * nw + (size_t)r * W + f] = z;
+            g.H[(l - 1) * nw + (size_t)r * W + f] = o;
         }
-        Z[(size_t)r * W + f] = z;
-        Hout[(size_t)r * W + f] = z > 0.f ? z : 0.f;
+    }
+    if (l < LAYERS) return;
+    __syncthreads();
+    if (threadIdx.x < kFwdRows && r0 + (int)threadIdx.x < n) {
+        float s = prm[OFF_BO];
+        for (int k = 0; k < W; ++k) s = __fmaf_rn(sO[threadIdx.x * W + k], prm[OFF_WO + k], s);
+        g.s[r0 + threadIdx.x] = s;
     }
 }
 
-// Logits, softmax and loss of one graph (one CTA of 256 threads):
-// s_i = h4_i . wo + bo; p_hat = softmax(s); L = -sum p_i log p_hat_i;
-// ds_i = p_hat_i sum(p) - p_i. Fixed-order reductions.
-__global__ void __launch_bounds__(256) softmax_loss_kernel(const float *__restrict__ H4, const float *__restrict__ prm,
-                                                           const double *__restrict__ p, int n,
-                                                           double *__restrict__ p_hat, float *__restrict__ ds,
-                                                           double *__restrict__ loss_acc, float *__restrict__ s_buf) {
+// Softmax and loss of a graph by a cluster of 8 CTAs: p_hat = softmax(s); L =
+// -sum p_i log p_hat_i; ds_i = p_hat_i sum(p) - p_i. The exponentials are FP64
+// (some 25 instructions, 40 ns each per scheduler: 38 us in one CTA at N =
+// 1000), so the CTAs share them; the first one forms the sums, in a fixed
+// order (its 256 threads over i, i + 256, ..., then the warps).
+constexpr int kSoftCtas = 8;
+__global__ void __cluster_dims__(kSoftCtas, 1, 1) __launch_bounds__(256)
+softmax_loss_kernel(const GnnDev *__restrict__ gs) {
     __shared__ double red[8];
+    __shared__ float redf[8];
     __shared__ double bc;
+    const GnnDev g = gs[blockIdx.y];
+    const int n = g.n, cta = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < n; i += blockDim.x) {
-        float s = prm[OFF_BO];
-        for (int k = 0; k < W; ++k) s = __fmaf_rn(H4[(size_t)i * W + k], prm[OFF_WO + k], s);
-        s_buf[i] = s;
-    }
-    __syncthreads();
-    auto bsum = [&](double v, bool is_max) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const double u = __shfl_xor_sync(0xffffffffu, v, o);
-            v = is_max ? fmax(v, u) : v + u;
-        }
+    const float *__restrict__ sb = g.s;
+    const double *__restrict__ p = g.p;
+    auto bsum = [&](double v) {
+        for (int o = 16; o > 0; o >>= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
         __syncthreads();
         if (lane == 0) red[warp] = v;
         __syncthreads();
         if (tid == 0) {
             double t = red[0];
-            for (int q = 1; q < 8; ++q) t = is_max ? fmax(t, red[q]) : t + red[q];
+            for (int q = 1; q < 8; ++q) t = t + red[q];
             bc = t;
         }
         __syncthreads();
         return bc;
     };
-    double mx = -INFINITY;
-    for (int i = tid; i < n; i += blockDim.x) mx = fmax(mx, (double)s_buf[i]);
-    mx = bsum(mx, true);
-    double se = 0.0, sp = 0.0;
-    for (int i = tid; i < n; i += blockDim.x) {
-        se += exp((double)s_buf[i] - mx);
-        sp += p ? p[i] : 0.0;
-    }
-    se = bsum(se, false);
-    sp = bsum(sp, false);
-    const double lse = mx + log(se);
-    double ls = 0.0;
-    for (int i = tid; i < n; i += blockDim.x) {
-        const double lp = (double)s_buf[i] - lse;
-        const double ph = exp(lp);
-        if (p_hat) p_hat[i] = ph;
-        if (p) {
-            ls -= p[i] * lp;
-            if (ds) ds[i] = (float)(ph * sp - p[i]);
+    auto barrier = [] {
+        __syncthreads();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    };
+    float mf = -INFINITY;
+    for (int i = tid; i < n; i += 256) mf = fmaxf(mf, sb[i]);
+    for (int o = 16; o > 0; o >>= 1) mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+    if (lane == 0) redf[warp] = mf;
+    __syncthreads();
+    for (int q = 0; q < 8; ++q) mf = fmaxf(mf, redf[q]);
+    const double mx = (double)mf;
+    for (int i = cta * 256 + tid; i < n; i += kSoftCtas * 256) g.e[i] = exp((double)sb[i] - mx);
+    barrier();
+    if (cta == 0) {
+        double se = 0.0, sp = 0.0;
+        for (int i = tid; i < n; i += 256) {
+            se += __ldcg(g.e + i);
+            sp += p ? p[i] : 0.0;
+        }
+        se = bsum(se);
+        sp = bsum(sp);
+        if (tid == 0) {
+            g.loss[1] = mx + log(se);
+            g.loss[2] = sp;
         }
     }
-    if (p) {
-        ls = bsum(ls, false);
-        if (tid == 0 && loss_acc) *loss_acc += ls;
+    barrier();
+    const double lse = __ldcg(g.loss + 1), sp = __ldcg(g.loss + 2);
+    for (int i = cta * 256 + tid; i < n; i += kSoftCtas * 256) {
+        const double ph = exp((double)sb[i] - lse);
+        g.p_hat[i] = ph;
+        if (p) g.ds[i] = (float)(ph * sp - p[i]);
+    }
+    if (p && cta == 0) {
+        double ls = 0.0;
+        for (int i = tid; i < n; i += 256) {
+            const double lp = (double)sb[i] - lse;
+            ls -= p[i] * lp;
+        }
+        ls = bsum(ls);
+        if (tid == 0) g.loss[0] = ls;
     }
 }
 
 // dH4 = ds wo^T (n x 64), and the partial sums of dwo = H4^T ds, dbo = sum ds
-// per block of kRowsWG rows.
-__global__ void __launch_bounds__(W) readout_bwd_kernel(const float *__restrict__ H4, const float *__restrict__ ds,
-                                                        const float *__restrict__ prm, int n, float *__restrict__ dH,
-                                                        float *__restrict__ part) {
-    const int f = threadIdx.x;
-    const int r0 = blockIdx.x * kRowsWG, r1 = min(n, r0 + kRowsWG);
-    float gw = 0.f, gb = 0.f;
-    const float wo = prm[OFF_WO + f];
-    for (int r = r0; r < r1; ++r) {
-        const float d = ds[r];
-        gw = __fmaf_rn(H4[(size_t)r * W + f], d, gw);
-        gb = __fadd_rn(gb, d);
-        dH[(size_t)r * W + f] = __fmul_rn(d, wo);
+// per block of kRowsWG rows (staged in shared memory: the sums run over rows).
+__global__ void __launch_bounds__(256) readout_bwd_kernel(const GnnDev *__restrict__ gs, const float *__restrict__ prm) {
+    __shared__ float sH[kRowsWG * W];
+    __shared__ float sd[kRowsWG];
+    const GnnDev g = gs[blockIdx.y];
+    if ((int)blockIdx.x >= g.nblk) return;
+    const int r0 = blockIdx.x * kRowsWG, rows = min(g.n - r0, kRowsWG);
+    const float *H4 = g.H + (size_t)(LAYERS - 1) * g.n * W;
+    for (int t = threadIdx.x; t < rows; t += blockDim.x) sd[t] = g.ds[r0 + t];
+    for (int t = threadIdx.x; t < rows * W; t += blockDim.x) sH[t] = H4[(size_t)r0 * W + t];
+    __syncthreads();
+    float *part = g.part + (size_t)blockIdx.x * kParams + OFF_WO;
+    if (threadIdx.x < W) {
+        float gw = 0.f;
+        for (int r = 0; r < rows; ++r) gw = __fmaf_rn(sH[r * W + threadIdx.x], sd[r], gw);
+        part[threadIdx.x] = gw;
+    } else if (threadIdx.x == W) {
+        float gb = 0.f;
+        for (int r = 0; r < rows; ++r) gb = __fadd_rn(gb, sd[r]);
+        part[W] = gb;
     }
-    part[(size_t)blockIdx.x * (W + 1) + f] = gw;
-    if (f == 0) part[(size_t)blockIdx.x * (W + 1) + W] = gb;
+    const float wo = prm[OFF_WO + (threadIdx.x & (W - 1))];
+    for (int t = threadIdx.x; t < rows * W; t += blockDim.x) g.dA[(size_t)r0 * W + t] = __fmul_rn(sd[t / W], wo);
 }
 
-// dZ = dH * [Z > 0] in place in dH; partial sums of dWs = H^T dZ,
-// dWn = M^T dZ, db = sum dZ per block of kRowsWG rows (din x 64 each).
-__global__ void __launch_bounds__(256) wgrad_kernel(const float *__restrict__ H, const float *__restrict__ M,
-                                                    const float *__restrict__ Z, float *__restrict__ dH, int n,
-                                                    int din, float *__restrict__ part) {
-    __shared__ float sdz[32 * W];
-    __shared__ float sH[32 * W], sM[32 * W];
-    const int per = 2 * din * W + W;
-    const int r0 = blockIdx.x * kRowsWG, r1 = min(n, r0 + kRowsWG);
-    // each thread owns 2*din*W/256 weight outputs (+ one bias for threads < W)
-    float acc[2 * W * W / 256];
-    const int nown = (2 * din * W) / 256;
-    for (int q = 0; q < nown; ++q) acc[q] = 0.f;
-    float accb = 0.f;
-    for (int rb = r0; rb < r1; rb += 32) {
-        const int rows = min(32, r1 - rb);
-        __syncthreads();
-        for (int t = threadIdx.x; t < 32 * W; t += blockDim.x) {
-            const int rr = t / W, f = t % W, r = rb + rr;
-            float dz = 0.f;
-            if (rr < rows) {
-                const size_t o = (size_t)r * W + f;
-                dz = Z[o] > 0.f ? dH[o] : 0.f;
-                dH[o] = dz;
-            }
-            sdz[t] = dz;
-        }
-        for (int t = threadIdx.x; t < 32 * din; t += blockDim.x) {
-            const int rr = t / din, k = t % din, r = rb + rr;
-            sH[t] = rr < rows ? H[(size_t)r * din + k] : 0.f;
-            sM[t] = rr < rows ? M[(size_t)r * din + k] : 0.f;
-        }
-        __syncthreads();
-        for (int q = 0; q < nown; ++q) {
-            const int idx = threadIdx.x + q * 256;  // 0 .. 2*din*W-1
-            const int which = idx / (din * W), rem = idx % (din * W), k = rem / W, f = rem % W;
-            const float *src = which == 0 ? sH : sM;
-            float a = acc[q];
-            for (int rr = 0; rr < rows; ++rr) a = __fmaf_rn(src[rr * din + k], sdz[rr * W + f], a);
-            acc[q] = a;
-        }
-        if (threadIdx.x < W)
-            for (int rr = 0; rr < rows; ++rr) accb = __fadd_rn(accb, sdz[rr * W + threadIdx.x]);
+// Partial sums of dWs = h^T dZ, dWn = M^T dZ, db = sum dZ of layer l per block
+// of kRowsWG rows, dZ = dH [Z > 0]. A CTA takes kWgCols columns of [h | M] (16
+// CTAs a block at width 64; one CTA a block left 8 of them on the chip at N =
+// 1000, 90 us) with the block's rows in shared memory.
+constexpr int kWgCols = 8;
+__global__ void __launch_bounds__(256) wgrad_kernel(const GnnDev *__restrict__ gs, int l, int odd) {
+    __shared__ float sdz[kRowsWG * W];
+    __shared__ float src[kRowsWG * kWgCols];
+    const GnnDev g = gs[blockIdx.y];
+    const int din = din_of(l), splits = 2 * din / kWgCols;
+    const int blk = blockIdx.x / splits, c0 = (blockIdx.x - blk * splits) * kWgCols;
+    if (blk >= g.nblk) return;
+    const int n = g.n, r0 = blk * kRowsWG, rows = min(n - r0, kRowsWG);
+    const size_t nw = (size_t)n * W;
+    const float *h = l == 1 ? g.x : g.H + (l - 2) * nw, *M = g.M + (l - 1) * nw, *Z = g.Z + (l - 1) * nw;
+    const float *dH = odd ? g.dB : g.dA;
+    for (int t = threadIdx.x; t < rows * W; t += blockDim.x) {
+        const size_t o = (size_t)r0 * W + t;
+        sdz[t] = Z[o] > 0.f ? dH[o] : 0.f;
     }
-    float *out = part + (size_t)blockIdx.x * per;
-    for (int q = 0; q < nown; ++q) out[threadIdx.x + q * 256] = acc[q];
-    if (threadIdx.x < W) out[2 * din * W + threadIdx.x] = accb;
+    for (int t = threadIdx.x; t < rows * kWgCols; t += blockDim.x) {
+        const int rr = t / kWgCols, c = c0 + t % kWgCols;
+        src[t] = (c < din ? h : M)[(size_t)(r0 + rr) * din + (c < din ? c : c - din)];
+    }
+    __syncthreads();
+    const int f = threadIdx.x & (W - 1), k = threadIdx.x >> 6;  // columns k and k + 4
+    float a0 = 0.f, a1 = 0.f;
+    for (int rr = 0; rr < rows; ++rr) {
+        const float dz = sdz[rr * W + f];
+        a0 = __fmaf_rn(src[rr * kWgCols + k], dz, a0);
+        a1 = __fmaf_rn(src[rr * kWgCols + k + 4], dz, a1);
+    }
+    float *out = g.part + (size_t)blk * kParams + off_ws(l);
+    out[(c0 + k) * W + f] = a0;
+    out[(c0 + k + 4) * W + f] = a1;
+    if (c0 == 0 && k == 0) {
+        float b = 0.f;
+        for (int rr = 0; rr < rows; ++rr) b = __fadd_rn(b, sdz[rr * W + f]);
+        out[2 * din * W + f] = b;
+    }
 }
 
-// grad[dst + t] += sum over blocks of part[b * per + t], in block order.
-__global__ void reduce_parts_kernel(const float *__restrict__ part, int nblocks, int per, float *__restrict__ grad) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= per) return;
-    float s = 0.f;
-    for (int b = 0; b < nblocks; ++b) s = __fadd_rn(s, part[(size_t)b * per + t]);
-    grad[t] = __fadd_rn(grad[t], s);
-}
-
-// dHs = dZ Ws^T, dT = dZ Wn^T (n x din): one thread per (row, k).
-__global__ void dense_bwd_kernel(const float *__restrict__ dZ, const float *__restrict__ prm, int l, int n,
-                                 float *__restrict__ dHs, float *__restrict__ dT) {
-    const int din = din_of(l);
-    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (t >= (size_t)n * din) return;
-    const int r = (int)(t / din), k = (int)(t % din);
-    const float *ws = prm + off_ws(l) + k * W, *wn = prm + off_wn(l) + k * W;
-    const float *dz = dZ + (size_t)r * W;
-    float a = 0.f, b = 0.f;
+// dHs = dZ Ws^T, dT = dZ Wn^T of layer l >= 2 (n x 64), dZ = dH [Z > 0]: 8
+// rows per CTA, the weights in shared memory (rows padded: the lanes read a
+// column).
+__global__ void __launch_bounds__(256) dense_bwd_kernel(const GnnDev *__restrict__ gs, const float *__restrict__ prm,
+                                                        int l, int odd) {
+    constexpr int LD = W + 1;
+    __shared__ float sS[W * LD], sN[W * LD], sdz[kFwdRows * W];
+    const GnnDev g = gs[blockIdx.y];
+    const int n = g.n, r0 = blockIdx.x * kFwdRows;
+    if (r0 >= n) return;
+    const float *dH = odd ? g.dB : g.dA;
+    float *dHs = odd ? g.dA : g.dB;
+    const float *Z = g.Z + (size_t)(l - 1) * n * W;
+    for (int t = threadIdx.x; t < W * W; t += blockDim.x) {
+        sS[(t / W) * LD + t % W] = prm[off_ws(l) + t];
+        sN[(t / W) * LD + t % W] = prm[off_wn(l) + t];
+    }
+    for (int t = threadIdx.x; t < kFwdRows * W; t += blockDim.x) {
+        const size_t o = (size_t)r0 * W + t;
+        sdz[t] = r0 + t / W < n && Z[o] > 0.f ? dH[o] : 0.f;
+    }
+    __syncthreads();
+    const int k = threadIdx.x & (W - 1), q = threadIdx.x >> 6;
+    float a0 = 0.f, b0 = 0.f, a1 = 0.f, b1 = 0.f;
     for (int f = 0; f < W; ++f) {
-        a = __fmaf_rn(dz[f], ws[f], a);
-        b = __fmaf_rn(dz[f], wn[f], b);
+        const float ws = sS[k * LD + f], wn = sN[k * LD + f], d0 = sdz[q * W + f], d1 = sdz[(q + 4) * W + f];
+        a0 = __fmaf_rn(d0, ws, a0);
+        b0 = __fmaf_rn(d0, wn, b0);
+        a1 = __fmaf_rn(d1, ws, a1);
+        b1 = __fmaf_rn(d1, wn, b1);
     }
-    dHs[t] = a;
-    dT[t] = b;
+    if (r0 + q < n) {
+        dHs[(size_t)(r0 + q) * W + k] = a0;
+        g.dT[(size_t)(r0 + q) * W + k] = b0;
+    }
+    if (r0 + q + 4 < n) {
+        dHs[(size_t)(r0 + q + 4) * W + k] = a1;
+        g.dT[(size_t)(r0 + q + 4) * W + k] = b1;
+    }
+}
+
+// dH of the layer below = dHs + P^T dT, one warp per row.
+__global__ void __launch_bounds__(256) spmm_bwd_kernel(const GnnDev *__restrict__ gs, int odd) {
+    const GnnDev g = gs[blockIdx.y];
+    const int lane = threadIdx.x & 31, i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (i >= g.n) return;
+    float a0, a1;
+    row_sum(g.tcol, g.tval, g.tptr[i], g.tptr[i + 1], g.dT, W, a0, a1);
+    float *y = (odd ? g.dA : g.dB) + (size_t)i * W;
+    y[lane] = __fadd_rn(y[lane], a0);
+    y[lane + 32] = __fadd_rn(y[lane + 32], a1);
+}
+
+// grad (zero first with `init`) += each graph's gradient (its blocks' partials
+// in order), graph after graph; *loss likewise.
+__global__ void reduce_kernel(const GnnDev *__restrict__ gs, int count, int init, float *__restrict__ grad,
+                              double *__restrict__ loss) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) {
+        double l = *loss;
+        for (int k = 0; k < count; ++k) l += gs[k].loss[0];
+        *loss = l;
+    }
+    if (t >= kParams) return;
+    float acc = init ? 0.f : grad[t];
+    for (int k = 0; k < count; ++k) {
+        const float *part = gs[k].part;
+        const int nblk = gs[k].nblk;
+        float s = 0.f;
+#pragma unroll 4
+        for (int b = 0; b < nblk; ++b) s = __fadd_rn(s, part[(size_t)b * kParams + t]);
+        acc = __fadd_rn(acc, s);
+    }
+    grad[t] = acc;
 }
 
 // Adam (bias-corrected) on the FP32 master weights; the forward copy keeps
@@ -383,13 +511,13 @@ struct qpr_gnn {
     cudaStream_t stream = nullptr;
     float *theta = nullptr, *fwd = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     int64_t adam_t = 0;
-    // per-graph device workspace (grown on demand)
-    int cap_n = 0, cap_nnz = 0;
-    float *x = nullptr, *H[5] = {}, *M[5] = {}, *Z[5] = {}, *dH = nullptr, *dHs = nullptr, *dT = nullptr;
-    float *ds = nullptr, *sbuf = nullptr, *part = nullptr;
-    int *pptr = nullptr, *pcol = nullptr, *tptr = nullptr, *tcol = nullptr;
-    float *pval = nullptr, *tval = nullptr;
-    double *p = nullptr, *p_hat = nullptr, *loss = nullptr;
+    // device memory grown on demand: the graphs, the group's descriptors, the
+    // workspace (sized in nodes and blocks of a group)
+    char *graphs = nullptr, *ws = nullptr;
+    size_t graphs_cap = 0, ws_cap = 0;
+    qpr::GnnDev *desc = nullptr;  // pinned: descriptors of the groups in flight
+    size_t desc_cap = 0;
+    double *loss = nullptr;
     std::vector<void *> bufs;
     std::string err;
 };
@@ -424,99 +552,152 @@ cudaError_t galloc(qpr_gnn *g, T **p, size_t count) {
     return e;
 }
 
-void free_ws(qpr_gnn *g) {
-    // workspace buffers are those allocated after the five parameter arrays
-    while (g->bufs.size() > 5) {
-        cudaFree(g->bufs.back());
-        g->bufs.pop_back();
-    }
-    g->cap_n = g->cap_nnz = 0;
-}
+size_t round16(size_t b) { return (b + 15) & ~(size_t)15; }
 
-qpr_status ensure_ws(qpr_gnn *g, int n, int nnz) {
-    if (n <= g->cap_n && nnz <= g->cap_nnz) return QPR_OK;
-    free_ws(g);
-    const int cn = std::max(n, g->cap_n), cz = std::max(nnz, g->cap_nnz);
-    GCUDA(g, galloc(g, &g->x, (size_t)cn * FIN));
-    for (int l = 1; l <= qpr::LAYERS; ++l) {
-        GCUDA(g, galloc(g, &g->H[l], (size_t)cn * W));
-        GCUDA(g, galloc(g, &g->M[l], (size_t)cn * W));
-        GCUDA(g, galloc(g, &g->Z[l], (size_t)cn * W));
+// Grow *buf to `bytes`.
+qpr_status grow(qpr_gnn *g, char **buf, size_t *cap, size_t bytes) {
+    if (bytes <= *cap) return QPR_OK;
+    if (*buf) {
+        GCUDA(g, cudaStreamSynchronize(g->stream));
+        cudaFree(*buf);
+        *buf = nullptr;
+        *cap = 0;
     }
-    GCUDA(g, galloc(g, &g->dH, (size_t)cn * W));
-    GCUDA(g, galloc(g, &g->dHs, (size_t)cn * W));
-    GCUDA(g, galloc(g, &g->dT, (size_t)cn * W));
-    GCUDA(g, galloc(g, &g->ds, cn));
-    GCUDA(g, galloc(g, &g->sbuf, cn));
-    const int nblk = (cn + qpr::kRowsWG - 1) / qpr::kRowsWG;
-    GCUDA(g, galloc(g, &g->part, (size_t)nblk * (2 * W * W + W)));
-    GCUDA(g, galloc(g, &g->pptr, cn + 1));
-    GCUDA(g, galloc(g, &g->tptr, cn + 1));
-    GCUDA(g, galloc(g, &g->pcol, cz));
-    GCUDA(g, galloc(g, &g->tcol, cz));
-    GCUDA(g, galloc(g, &g->pval, cz));
-    GCUDA(g, galloc(g, &g->tval, cz));
-    GCUDA(g, galloc(g, &g->p, cn));
-    GCUDA(g, galloc(g, &g->p_hat, cn));
-    GCUDA(g, galloc(g, &g->loss, 1));
-    g->cap_n = cn;
-    g->cap_nnz = cz;
+    GCUDA(g, cudaMalloc((void **)buf, bytes));
+    *cap = bytes;
     return QPR_OK;
 }
 
-qpr_status upload_graph(qpr_gnn *g, const qpr::HostGraph &hg, const double *p) {
-    const int n = hg.n, nnz = (int)hg.pcol.size();
-    qpr_status st = ensure_ws(g, n, std::max(nnz, 1));
+// Bytes of a graph in device memory, and the image of it with the pointers
+// that it has at `dev`.
+size_t graph_bytes(const qpr::HostGraph &hg) {
+    const size_t n = hg.n, nnz = hg.pcol.size();
+    return round16(hg.x.size() * 4) + 2 * round16((n + 1) * 4) + 4 * round16(nnz * 4) + round16(n * 8);
+}
+void put_graph(const qpr::HostGraph &hg, const double *p, char *host, char *dev, qpr::GnnDev *d) {
+    size_t at = 0;
+    auto put = [&](const void *src, size_t bytes) {
+        if (bytes) memcpy(host + at, src, bytes);
+        char *q = dev + at;
+        at += round16(bytes);
+        return q;
+    };
+    d->n = hg.n;
+    d->nblk = (hg.n + qpr::kRowsWG - 1) / qpr::kRowsWG;
+    d->x = (const float *)put(hg.x.data(), hg.x.size() * 4);
+    d->pptr = (const int *)put(hg.pptr.data(), hg.pptr.size() * 4);
+    d->tptr = (const int *)put(hg.tptr.data(), hg.tptr.size() * 4);
+    d->pcol = (const int *)put(hg.pcol.data(), hg.pcol.size() * 4);
+    d->tcol = (const int *)put(hg.tcol.data(), hg.tcol.size() * 4);
+    d->pval = (const float *)put(hg.pval.data(), hg.pval.size() * 4);
+    d->tval = (const float *)put(hg.tval.data(), hg.tval.size() * 4);
+    d->p = p ? (const double *)put(p, (size_t)hg.n * 8) : nullptr;
+}
+
+// Bytes of workspace of one graph.
+size_t ws_bytes(int n) {
+    const size_t nw = (size_t)n * W, nblk = (n + qpr::kRowsWG - 1) / qpr::kRowsWG;
+    return round16((15 * nw + 2 * (size_t)n) * 4) + 2 * round16((size_t)n * 8) + round16(nblk * qpr::kParams * 4) + 32;
+}
+void place_ws(char *at, qpr::GnnDev *d) {
+    const size_t n = d->n, nw = n * W;
+    float *f = (float *)at;
+    d->H = f;
+    d->M = f + 4 * nw;
+    d->Z = f + 8 * nw;
+    d->dA = f + 12 * nw;
+    d->dB = f + 13 * nw;
+    d->dT = f + 14 * nw;
+    d->s = f + 15 * nw;
+    d->ds = d->s + n;
+    at += round16((15 * nw + 2 * n) * 4);
+    d->e = (double *)at;
+    at += round16(n * 8);
+    d->p_hat = (double *)at;
+    at += round16(n * 8);
+    d->part = (float *)at;
+    at += round16((size_t)d->nblk * qpr::kParams * 4);
+    d->loss = (double *)at;
+}
+
+// Room for `count` pinned descriptors.
+qpr_status grow_desc(qpr_gnn *g, size_t count) {
+    if (count <= g->desc_cap) return QPR_OK;
+    GCUDA(g, cudaStreamSynchronize(g->stream));
+    cudaFreeHost(g->desc);
+    g->desc = nullptr;
+    g->desc_cap = 0;
+    GCUDA(g, cudaMallocHost((void **)&g->desc, count * sizeof(qpr::GnnDev)));
+    g->desc_cap = count;
+    return QPR_OK;
+}
+
+// The workspace of a group (count descriptors at grp, pinned and left alone
+// until the stream has been waited for) and its descriptors behind it on the
+// device.
+qpr_status place_group(qpr_gnn *g, qpr::GnnDev *grp, size_t count, qpr::GnnDev **dev) {
+    size_t bytes = 0;
+    for (size_t k = 0; k < count; ++k) bytes += ws_bytes(grp[k].n);
+    const qpr_status st = grow(g, &g->ws, &g->ws_cap, bytes + count * sizeof(qpr::GnnDev));
     if (st != QPR_OK) return st;
-    cudaStream_t s = g->stream;
-    GCUDA(g, cudaMemcpyAsync(g->x, hg.x.data(), hg.x.size() * sizeof(float), cudaMemcpyHostToDevice, s));
-    GCUDA(g, cudaMemcpyAsync(g->pptr, hg.pptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, s));
-    GCUDA(g, cudaMemcpyAsync(g->tptr, hg.tptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice, s));
-    if (nnz > 0) {
-        GCUDA(g, cudaMemcpyAsync(g->pcol, hg.pcol.data(), nnz * sizeof(int), cudaMemcpyHostToDevice, s));
-        GCUDA(g, cudaMemcpyAsync(g->tcol, hg.tcol.data(), nnz * sizeof(int), cudaMemcpyHostToDevice, s));
-        GCUDA(g, cudaMemcpyAsync(g->pval, hg.pval.data(), nnz * sizeof(float), cudaMemcpyHostToDevice, s));
-        GCUDA(g, cudaMemcpyAsync(g->tval, hg.tval.data(), nnz * sizeof(float), cudaMemcpyHostToDevice, s));
+    size_t at = 0;
+    for (size_t k = 0; k < count; ++k) {
+        place_ws(g->ws + at, &grp[k]);
+        at += ws_bytes(grp[k].n);
     }
-    if (p) GCUDA(g, cudaMemcpyAsync(g->p, p, n * sizeof(double), cudaMemcpyHostToDevice, s));
-    // the host vectors die with the caller: finish the copies now
-    GCUDA(g, cudaStreamSynchronize(s));
+    *dev = (qpr::GnnDev *)(g->ws + at);
+    GCUDA(g, cudaMemcpyAsync(*dev, grp, count * sizeof(qpr::GnnDev), cudaMemcpyHostToDevice, g->stream));
     return QPR_OK;
 }
 
-// Forward pass (and, with a target, loss and backward into g->grad).
-void enqueue_pass(qpr_gnn *g, int n, bool with_target, bool backward) {
+// Forward pass of a group (and, with targets, loss and backward into g->grad,
+// zeroed first with `init`).
+void enqueue_pass(qpr_gnn *g, const qpr::GnnDev *dev, int count, int maxn, bool backward, bool init) {
     cudaStream_t s = g->stream;
-    const int wpb = 8, rows_blocks = (n + wpb - 1) / wpb;
-    const float *h = g->x;
-    g->H[0] = g->x;
-    for (int l = 1; l <= qpr::LAYERS; ++l) {
-        const int din = qpr::din_of(l);
-        qpr::spmm_rows_kernel<<<rows_blocks, 256, 0, s>>>(g->pptr, g->pcol, g->pval, h, g->M[l], n, din, 0);
-        qpr::dense_fwd_kernel<<<(n + 31) / 32, 256, 0, s>>>(h, g->M[l], g->fwd, l, n, g->Z[l], g->H[l]);
-        h = g->H[l];
-    }
-    qpr::softmax_loss_kernel<<<1, 256, 0, s>>>(g->H[qpr::LAYERS], g->fwd, with_target ? g->p : nullptr, n, g->p_hat,
-                                             g->ds, g->loss, g->sbuf);
+    const dim3 rows((maxn + qpr::kFwdRows - 1) / qpr::kFwdRows, count);
+    for (int l = 1; l <= qpr::LAYERS; ++l) qpr::layer_fwd_kernel<<<rows, 256, 0, s>>>(dev, g->fwd, l);
+    qpr::softmax_loss_kernel<<<dim3(qpr::kSoftCtas, count), 256, 0, s>>>(dev);
     if (!backward) return;
-    const int nblk = (n + qpr::kRowsWG - 1) / qpr::kRowsWG;
-    qpr::readout_bwd_kernel<<<nblk, W, 0, s>>>(g->H[qpr::LAYERS], g->ds, g->fwd, n, g->dH, g->part);
-    qpr::reduce_parts_kernel<<<1, 128, 0, s>>>(g->part, nblk, W + 1, g->grad + qpr::OFF_WO);
+    const int nblk = (maxn + qpr::kRowsWG - 1) / qpr::kRowsWG;
+    qpr::readout_bwd_kernel<<<dim3(nblk, count), 256, 0, s>>>(dev, g->fwd);
+    int odd = 0;  // the output gradient of the layer is in dB
     for (int l = qpr::LAYERS; l >= 1; --l) {
-        const int din = qpr::din_of(l);
-        const float *hin = (l == 1) ? g->x : g->H[l - 1];
-        qpr::wgrad_kernel<<<nblk, 256, 0, s>>>(hin, g->M[l], g->Z[l], g->dH, n, din, g->part);
-        const int per = 2 * din * W + W;
-        qpr::reduce_parts_kernel<<<(per + 255) / 256, 256, 0, s>>>(g->part, nblk, per, g->grad + qpr::off_ws(l));
+        const int splits = 2 * qpr::din_of(l) / qpr::kWgCols;
+        qpr::wgrad_kernel<<<dim3(nblk * splits, count), 256, 0, s>>>(dev, l, odd);
         if (l > 1) {
-            const size_t tot = (size_t)n * din;
-            qpr::dense_bwd_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(g->dH, g->fwd, l, n, g->dHs, g->dT);
-            // dH_{l-1} = dHs + P^T dT
-            qpr::spmm_rows_kernel<<<rows_blocks, 256, 0, s>>>(g->tptr, g->tcol, g->tval, g->dT, g->dHs, n, din, 1);
-            std::swap(g->dH, g->dHs);
+            qpr::dense_bwd_kernel<<<rows, 256, 0, s>>>(dev, g->fwd, l, odd);
+            qpr::spmm_bwd_kernel<<<dim3((maxn + 7) / 8, count), 256, 0, s>>>(dev, odd);
+            odd ^= 1;
         }
     }
+    qpr::reduce_kernel<<<(qpr::kParams + 127) / 128, 128, 0, s>>>(dev, count, init ? 1 : 0, g->grad, g->loss);
 }
+
+// One graph, as predict and loss_grad run it.
+qpr_status single_pass(qpr_gnn *g, const qpr::HostGraph &hg, const double *p, bool backward, qpr::GnnDev *out) {
+    const size_t bytes = graph_bytes(hg);
+    qpr_status st = grow(g, &g->graphs, &g->graphs_cap, bytes);
+    if (st == QPR_OK) st = grow_desc(g, 1);
+    if (st != QPR_OK) return st;
+    std::vector<char> img(bytes);
+    put_graph(hg, p, img.data(), g->graphs, g->desc);
+    GCUDA(g, cudaMemcpyAsync(g->graphs, img.data(), bytes, cudaMemcpyHostToDevice, g->stream));
+    qpr::GnnDev *dev = nullptr;
+    st = place_group(g, g->desc, 1, &dev);
+    if (st != QPR_OK) return st;
+    if (backward) GCUDA(g, cudaMemsetAsync(g->loss, 0, sizeof(double), g->stream));
+    enqueue_pass(g, dev, 1, hg.n, backward, true);
+    *out = g->desc[0];
+    // `img` and the descriptor are free again after this
+    GCUDA(g, cudaStreamSynchronize(g->stream));
+    return QPR_OK;
+}
+
+// Nodes of a group at most (unless one graph has more): 250 MB of workspace.
+constexpr int kGroupNodes = 65536;
+// The training set stays on the device up to this size; beyond it every group
+// is uploaded for its pass.
+constexpr size_t kResidentBytes = (size_t)2 << 30;
 
 }  // namespace
 
@@ -531,6 +712,9 @@ void qpr_gnn_destroy(qpr_gnn *g) {
     cudaSetDevice(g->device);
     if (g->stream) cudaStreamSynchronize(g->stream);
     for (void *p : g->bufs) cudaFree(p);
+    cudaFree(g->graphs);
+    cudaFree(g->ws);
+    cudaFreeHost(g->desc);
     if (g->stream) cudaStreamDestroy(g->stream);
     cudaGetLastError();
     if (prev >= 0) cudaSetDevice(prev);
@@ -559,7 +743,7 @@ qpr_status qpr_gnn_create(qpr_gnn **out, uint64_t seed, int32_t device) {
     const int P = qpr::kParams;
     if (galloc(g, &g->theta, P) != cudaSuccess || galloc(g, &g->fwd, P) != cudaSuccess ||
         galloc(g, &g->grad, P) != cudaSuccess || galloc(g, &g->m, P) != cudaSuccess ||
-        galloc(g, &g->v, P) != cudaSuccess || cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess)
+        galloc(g, &g->v, P) != cudaSuccess || galloc(g, &g->loss, 1) != cudaSuccess || cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking) != cudaSuccess)
         return bail(gnn_fail(nullptr, QPR_E_OOM, "device allocation failed"));
     // Glorot-uniform weights from splitmix64(seed), zero biases
     std::vector<float> th(P, 0.f);
@@ -611,10 +795,10 @@ qpr_status qpr_gnn_predict(qpr_gnn *g, int64_t n, int64_t m, const int64_t *src,
     std::string e;
     qpr_status st = qpr::build_graph(n, m, src, dst, w, alpha, omega, hg, e);
     if (st != QPR_OK) return gnn_fail(g, st, e);
-    st = upload_graph(g, hg, nullptr);
+    qpr::GnnDev d;
+    st = single_pass(g, hg, nullptr, false, &d);
     if (st != QPR_OK) return st;
-    enqueue_pass(g, (int)n, false, false);
-    GCUDA(g, cudaMemcpyAsync(p_hat, g->p_hat, n * sizeof(double), cudaMemcpyDefault, g->stream));
+    GCUDA(g, cudaMemcpyAsync(p_hat, d.p_hat, n * sizeof(double), cudaMemcpyDefault, g->stream));
     GCUDA(g, cudaStreamSynchronize(g->stream));
     GCUDA(g, cudaGetLastError());
     return QPR_OK;
@@ -627,11 +811,9 @@ qpr_status qpr_gnn_loss_grad(qpr_gnn *g, const qpr_gnn_sample *smp, double alpha
     std::string e;
     qpr_status st = qpr::build_graph(smp->n, smp->m, smp->src, smp->dst, smp->w, alpha, smp->omega, hg, e);
     if (st != QPR_OK) return gnn_fail(g, st, e);
-    st = upload_graph(g, hg, smp->p);
+    qpr::GnnDev d;
+    st = single_pass(g, hg, smp->p, true, &d);
     if (st != QPR_OK) return st;
-    GCUDA(g, cudaMemsetAsync(g->grad, 0, qpr::kParams * sizeof(float), g->stream));
-    GCUDA(g, cudaMemsetAsync(g->loss, 0, sizeof(double), g->stream));
-    enqueue_pass(g, (int)smp->n, true, true);
     if (loss) GCUDA(g, cudaMemcpyAsync(loss, g->loss, sizeof(double), cudaMemcpyDeviceToHost, g->stream));
     if (grad) GCUDA(g, cudaMemcpyAsync(grad, g->grad, qpr::kParams * sizeof(float), cudaMemcpyDeviceToHost, g->stream));
     GCUDA(g, cudaStreamSynchronize(g->stream));
@@ -651,13 +833,35 @@ qpr_status qpr_gnn_train(qpr_gnn *g, int64_t count, const qpr_gnn_sample *sample
                                                samples[i].w, alpha, samples[i].omega, hg[i], e);
         if (st != QPR_OK) return gnn_fail(g, st, "sample " + std::to_string(i) + ": " + e);
     }
-    {
-        int maxn = 2, maxz = 1;
-        for (const qpr::HostGraph &h : hg) {
-            maxn = std::max(maxn, h.n);
-            maxz = std::max(maxz, (int)h.pcol.size());
+    // the graphs: all on the device, or a group at a time
+    size_t total = 0;
+    for (const qpr::HostGraph &h : hg) total += graph_bytes(h);
+    const bool resident = total <= kResidentBytes;
+    std::vector<qpr::GnnDev> graphs((size_t)count);
+    std::vector<char> img;
+    auto upload = [&](const std::vector<int64_t> &ids) -> qpr_status {
+        size_t bytes = 0;
+        for (int64_t i : ids) bytes += graph_bytes(hg[i]);
+        const qpr_status st = grow(g, &g->graphs, &g->graphs_cap, bytes);
+        if (st != QPR_OK) return st;
+        img.resize(bytes);
+        size_t at = 0;
+        for (int64_t i : ids) {
+            put_graph(hg[i], samples[i].p, img.data() + at, g->graphs + at, &graphs[i]);
+            at += graph_bytes(hg[i]);
         }
-        const qpr_status st = ensure_ws(g, maxn, maxz);
+        GCUDA(g, cudaMemcpyAsync(g->graphs, img.data(), bytes, cudaMemcpyHostToDevice, g->stream));
+        GCUDA(g, cudaStreamSynchronize(g->stream));  // img is reused
+        return QPR_OK;
+    };
+    if (resident) {
+        std::vector<int64_t> all((size_t)count);
+        for (int64_t i = 0; i < count; ++i) all[i] = i;
+        const qpr_status st = upload(all);
+        if (st != QPR_OK) return st;
+    }
+    {
+        const qpr_status st = grow_desc(g, (size_t)count);
         if (st != QPR_OK) return st;
     }
     std::vector<int64_t> order((size_t)count);
@@ -669,12 +873,25 @@ qpr_status qpr_gnn_train(qpr_gnn *g, int64_t count, const qpr_gnn_sample *sample
         GCUDA(g, cudaMemsetAsync(g->loss, 0, sizeof(double), g->stream));
         for (int64_t b0 = 0; b0 < count; b0 += batch) {
             const int64_t b1i = std::min<int64_t>(count, b0 + batch);
-            GCUDA(g, cudaMemsetAsync(g->grad, 0, qpr::kParams * sizeof(float), g->stream));
-            for (int64_t k = b0; k < b1i; ++k) {
-                const int64_t i = order[k];
-                qpr_status st = upload_graph(g, hg[i], samples[i].p);
+            for (int64_t k = b0; k < b1i;) {
+                std::vector<int64_t> ids;
+                int nodes = 0, maxn = 0;
+                for (; k < b1i && ids.size() < 4096 && (ids.empty() || nodes + hg[order[k]].n <= kGroupNodes); ++k) {
+                    ids.push_back(order[k]);
+                    nodes += hg[order[k]].n;
+                    maxn = std::max(maxn, hg[order[k]].n);
+                }
+                const bool init = (int64_t)ids.size() == k - b0;  // the batch's first group
+                if (!resident) {
+                    const qpr_status st = upload(ids);
+                    if (st != QPR_OK) return st;
+                }
+                // an epoch uses each descriptor slot once and ends with a wait
+                qpr::GnnDev *grp = g->desc + (k - (int64_t)ids.size()), *dev = nullptr;
+                for (size_t q = 0; q < ids.size(); ++q) grp[q] = graphs[ids[q]];
+                const qpr_status st = place_group(g, grp, ids.size(), &dev);
                 if (st != QPR_OK) return st;
-                enqueue_pass(g, hg[i].n, true, true);
+                enqueue_pass(g, dev, (int)ids.size(), maxn, true, init);
             }
             ++g->adam_t;
             const float c1 = 1.f - powf(b1, (float)g->adam_t), c2 = 1.f - powf(b2, (float)g->adam_t);
