@@ -17,6 +17,7 @@
 // cores to matter, so they run on the FP32 pipe with the BF16-rounded weights
 // staged in shared memory; every reduction (weight gradients, softmax) is in
 // fixed order, so training is bitwise reproducible.
+#include <limits.h>
 #include <math.h>
 #include <string.h>
 
@@ -410,30 +411,105 @@ struct HostGraph {
     std::vector<float> x;                        // n x FIN
     std::vector<int> pptr, pcol, tptr, tcol;     // P and P^T in CSR
     std::vector<float> pval, tval;
+    // the PageRank feature (x_6) is formed on the device from these (up to
+    // kPrClusterMaxN nodes; above, here)
+    bool device_pr = false;
+    double alpha = 0.0;
+    std::vector<int> sptr, scol;
+    std::vector<double> sval;
+    std::vector<unsigned char> dang;
 };
 
-// Features and aggregation of one graph (see the file header).
+constexpr int kPrIters = 200, kPrFeature = 6;
+
+// Below this many entries and nodes a lone graph's power iteration is faster
+// here (measured: N = 100 230 us a call, N = 200 470) than in a cluster (3 us an iteration
+// whatever the graph: N = 130 to 200 540 to 610); the graphs of a training set run
+// side by side there.
+constexpr int kPrHostWork = 2200;
+
+// Features and aggregation of one graph (see the file header); one of many?
 qpr_status build_graph(int64_t n, int64_t m, const int64_t *src, const int64_t *dst, const double *w, double alpha,
-                       double omega, HostGraph &out, std::string &err) {
+                       double omega, HostGraph &out, std::string &err, bool many = false) {
     HostOps h;
-    const qpr_status st = assemble_host(n, m, src, dst, w, QPR_HDIAG_ZERO, h, err);
+    const qpr_status st = assemble_host(n, m, src, dst, w, QPR_HDIAG_ZERO, h, err, false);
     if (st != QPR_OK) return st;
-    // A entries (i, j, a) from the CSR of S: A_ij = S_ij outDeg(j)
-    struct E { int i, j; double a; };
-    std::vector<E> ents;
-    for (int64_t i = 0; i < n; ++i)
-        for (int q = h.sptr[i]; q < h.sptr[i + 1]; ++q) ents.push_back({(int)i, h.scol[q], h.sval[q] * h.outdeg[h.scol[q]]});
+    // A entries (i, j, a) from the CSR of S: A_ij = S_ij outDeg(j); and of
+    // the transpose, columns in order
+    const size_t nnz = h.scol.size();
+    std::vector<double> av(nnz), tv(nnz);
+    std::vector<int> tp(n + 1, 0), tc(nnz);
     std::vector<double> instr(n, 0.0);
-    std::vector<int> indeg(n, 0), outdeg_cnt(n, 0);
-    for (const E &e : ents) {
-        instr[e.i] += e.a;
-        indeg[e.i] += 1;
-        outdeg_cnt[e.j] += 1;
+    for (int64_t i = 0; i < n; ++i)
+        for (int q = h.sptr[i]; q < h.sptr[i + 1]; ++q) {
+            av[q] = h.sval[q] * h.outdeg[h.scol[q]];
+            instr[i] += av[q];
+            tp[h.scol[q] + 1] += 1;
+        }
+    for (int64_t i = 0; i < n; ++i) tp[i + 1] += tp[i];
+    {
+        std::vector<int> at(tp.begin(), tp.end() - 1);
+        for (int64_t i = 0; i < n; ++i)
+            for (int q = h.sptr[i]; q < h.sptr[i + 1]; ++q) {
+                const int t = at[h.scol[q]]++;
+                tc[t] = (int)i;
+                tv[t] = av[q];
+            }
+    }
+    out.n = (int)n;
+    out.x.assign((size_t)n * FIN, 0.f);
+    for (int64_t i = 0; i < n; ++i) {
+        float *x = &out.x[(size_t)i * FIN];
+        x[0] = 1.f;
+        x[1] = (float)omega;
+        x[2] = (float)log1p(instr[i]);
+        x[3] = (float)log1p(h.outdeg[i]);
+        x[4] = (float)log1p((double)(h.sptr[i + 1] - h.sptr[i]));
+        x[5] = (float)log1p((double)(tp[i + 1] - tp[i]));
+        x[7] = h.dang[i] ? 1.f : 0.f;
+    }
+    // B = A + A^T row by row (the two sorted rows merged), P = B
+    // row-normalised; B is symmetric, so P^T has its pattern
+    out.pptr.assign(n + 1, 0);
+    out.pcol.reserve(2 * nnz);
+    std::vector<double> bv, rs(n, 0.0);
+    bv.reserve(2 * nnz);
+    for (int64_t i = 0; i < n; ++i) {
+        int qa = h.sptr[i], qt = tp[i];
+        while (qa < h.sptr[i + 1] || qt < tp[i + 1]) {
+            const int ja = qa < h.sptr[i + 1] ? h.scol[qa] : INT_MAX, jt = qt < tp[i + 1] ? tc[qt] : INT_MAX;
+            const int j = std::min(ja, jt);
+            double v = 0.0;
+            if (ja == j) v = av[qa++];
+            if (jt == j) v += tv[qt++];
+            out.pcol.push_back(j);
+            bv.push_back(v);
+            rs[i] += v;
+        }
+        out.pptr[i + 1] = (int)out.pcol.size();
+    }
+    out.tptr = out.pptr;
+    out.tcol = out.pcol;
+    out.pval.resize(bv.size());
+    out.tval.resize(bv.size());
+    for (int64_t i = 0; i < n; ++i)
+        for (int q = out.pptr[i]; q < out.pptr[i + 1]; ++q) {
+            out.pval[q] = (float)(bv[q] / rs[i]);
+            out.tval[q] = (float)(bv[q] / rs[out.pcol[q]]);
+        }
+    out.device_pr = n <= kPrClusterMaxN && (many || (int64_t)nnz + 2 * n > kPrHostWork);
+    out.alpha = alpha;
+    if (out.device_pr) {
+        out.sptr = std::move(h.sptr);
+        out.scol = std::move(h.scol);
+        out.sval = std::move(h.sval);
+        out.dang = std::move(h.dang);
+        return QPR_OK;
     }
     // classical PageRank: pi <- G pi, renormalised, 200 steps from uniform
     std::vector<double> pi(n, 1.0 / (double)n), nx(n);
     const double inv_nm1 = 1.0 / (double)(n - 1);
-    for (int it = 0; it < 200; ++it) {
+    for (int it = 0; it < kPrIters; ++it) {
         double P = 0.0, D = 0.0;
         for (int64_t j = 0; j < n; ++j) {
             P += pi[j];
@@ -449,50 +525,7 @@ qpr_status build_graph(int64_t n, int64_t m, const int64_t *src, const int64_t *
         }
         for (int64_t i = 0; i < n; ++i) pi[i] = nx[i] / tot;
     }
-    out.n = (int)n;
-    out.x.assign((size_t)n * FIN, 0.f);
-    for (int64_t i = 0; i < n; ++i) {
-        float *x = &out.x[(size_t)i * FIN];
-        x[0] = 1.f;
-        x[1] = (float)omega;
-        x[2] = (float)log1p(instr[i]);
-        x[3] = (float)log1p(h.outdeg[i]);
-        x[4] = (float)log1p((double)indeg[i]);
-        x[5] = (float)log1p((double)outdeg_cnt[i]);
-        x[6] = (float)log((double)n * pi[i]);
-        x[7] = h.dang[i] ? 1.f : 0.f;
-    }
-    // B = A + A^T, P = B row-normalised, and its transpose
-    std::vector<E> b;
-    for (const E &e : ents) {
-        b.push_back({e.i, e.j, e.a});
-        b.push_back({e.j, e.i, e.a});
-    }
-    std::sort(b.begin(), b.end(), [](const E &x, const E &y) { return x.i != y.i ? x.i < y.i : x.j < y.j; });
-    std::vector<E> bu;
-    for (const E &e : b) {
-        if (!bu.empty() && bu.back().i == e.i && bu.back().j == e.j) bu.back().a += e.a;
-        else bu.push_back(e);
-    }
-    std::vector<double> rs(n, 0.0);
-    for (const E &e : bu) rs[e.i] += e.a;
-    out.pptr.assign(n + 1, 0);
-    for (const E &e : bu) {
-        out.pcol.push_back(e.j);
-        out.pval.push_back((float)(e.a / rs[e.i]));
-        out.pptr[e.i + 1]++;
-    }
-    for (int64_t i = 0; i < n; ++i) out.pptr[i + 1] += out.pptr[i];
-    std::vector<E> t;
-    for (size_t q = 0; q < bu.size(); ++q) t.push_back({bu[q].j, bu[q].i, (double)out.pval[q]});
-    std::sort(t.begin(), t.end(), [](const E &x, const E &y) { return x.i != y.i ? x.i < y.i : x.j < y.j; });
-    out.tptr.assign(n + 1, 0);
-    for (const E &e : t) {
-        out.tcol.push_back(e.j);
-        out.tval.push_back((float)e.a);
-        out.tptr[e.i + 1]++;
-    }
-    for (int64_t i = 0; i < n; ++i) out.tptr[i + 1] += out.tptr[i];
+    for (int64_t i = 0; i < n; ++i) out.x[(size_t)i * FIN + kPrFeature] = (float)log((double)n * pi[i]);
     return QPR_OK;
 }
 
@@ -568,13 +601,17 @@ qpr_status grow(qpr_gnn *g, char **buf, size_t *cap, size_t bytes) {
     return QPR_OK;
 }
 
-// Bytes of a graph in device memory, and the image of it with the pointers
-// that it has at `dev`.
+// Bytes of a graph in device memory (with what its PageRank feature is
+// formed from, until it has one), and the image of it with the pointers that
+// it has at `dev`; a PageRank job goes to `jobs`.
 size_t graph_bytes(const qpr::HostGraph &hg) {
     const size_t n = hg.n, nnz = hg.pcol.size();
-    return round16(hg.x.size() * 4) + 2 * round16((n + 1) * 4) + 4 * round16(nnz * 4) + round16(n * 8);
+    size_t b = round16(hg.x.size() * 4) + 2 * round16((n + 1) * 4) + 4 * round16(nnz * 4) + round16(n * 8);
+    if (hg.device_pr) b += round16((n + 1) * 4) + round16(hg.scol.size() * 4) + round16(hg.sval.size() * 8) + round16(n);
+    return b;
 }
-void put_graph(const qpr::HostGraph &hg, const double *p, char *host, char *dev, qpr::GnnDev *d) {
+void put_graph(const qpr::HostGraph &hg, const double *p, char *host, char *dev, qpr::GnnDev *d,
+               std::vector<qpr::PrJob> &jobs) {
     size_t at = 0;
     auto put = [&](const void *src, size_t bytes) {
         if (bytes) memcpy(host + at, src, bytes);
@@ -592,6 +629,49 @@ void put_graph(const qpr::HostGraph &hg, const double *p, char *host, char *dev,
     d->pval = (const float *)put(hg.pval.data(), hg.pval.size() * 4);
     d->tval = (const float *)put(hg.tval.data(), hg.tval.size() * 4);
     d->p = p ? (const double *)put(p, (size_t)hg.n * 8) : nullptr;
+    if (!hg.device_pr) return;
+    qpr::PrJob j{};
+    j.n = hg.n;
+    j.dangling = QPR_DANGLING_F;
+    j.alpha = hg.alpha;
+    j.s_ptr = (const int *)put(hg.sptr.data(), hg.sptr.size() * 4);
+    j.s_col = (const int *)put(hg.scol.data(), hg.scol.size() * 4);
+    j.s_val = (const double *)put(hg.sval.data(), hg.sval.size() * 8);
+    j.dang = (const unsigned char *)put(hg.dang.data(), hg.dang.size());
+    j.feature = const_cast<float *>(d->x) + qpr::kPrFeature;
+    j.stride = qpr::FIN;
+    jobs.push_back(j);
+}
+
+// Upload graphs (targets p[i], or null) into g->graphs, their descriptors to
+// graphs[i], and form the PageRank features of those that have none. Returns
+// with `img` free again.
+qpr_status upload_graphs(qpr_gnn *g, const std::vector<const qpr::HostGraph *> &hg, const std::vector<const double *> &p,
+                         const std::vector<qpr::GnnDev *> &graphs, std::vector<char> &img) {
+    size_t bytes = 0;
+    int maxn = 0;
+    for (const qpr::HostGraph *h : hg) {
+        bytes += graph_bytes(*h);
+        if (h->device_pr) maxn = std::max(maxn, h->n);
+    }
+    const size_t all = bytes + hg.size() * sizeof(qpr::PrJob);
+    const qpr_status st = grow(g, &g->graphs, &g->graphs_cap, all);
+    if (st != QPR_OK) return st;
+    if (img.size() < all) img.resize(all);
+    std::vector<qpr::PrJob> jobs;
+    size_t at = 0;
+    for (size_t k = 0; k < hg.size(); ++k) {
+        put_graph(*hg[k], p[k], img.data() + at, g->graphs + at, graphs[k], jobs);
+        at += graph_bytes(*hg[k]);
+    }
+    if (!jobs.empty()) memcpy(img.data() + bytes, jobs.data(), jobs.size() * sizeof(qpr::PrJob));
+    GCUDA(g, cudaMemcpyAsync(g->graphs, img.data(), bytes + jobs.size() * sizeof(qpr::PrJob), cudaMemcpyHostToDevice,
+                             g->stream));
+    if (!jobs.empty())
+        GCUDA(g, qpr::pagerank_jobs((const qpr::PrJob *)(g->graphs + bytes), (int)jobs.size(), maxn, qpr::kPrIters,
+                                    g->stream));
+    GCUDA(g, cudaStreamSynchronize(g->stream));
+    return QPR_OK;
 }
 
 // Bytes of workspace of one graph.
@@ -675,20 +755,18 @@ void enqueue_pass(qpr_gnn *g, const qpr::GnnDev *dev, int count, int maxn, bool 
 
 // One graph, as predict and loss_grad run it.
 qpr_status single_pass(qpr_gnn *g, const qpr::HostGraph &hg, const double *p, bool backward, qpr::GnnDev *out) {
-    const size_t bytes = graph_bytes(hg);
-    qpr_status st = grow(g, &g->graphs, &g->graphs_cap, bytes);
-    if (st == QPR_OK) st = grow_desc(g, 1);
+    qpr_status st = grow_desc(g, 1);
     if (st != QPR_OK) return st;
-    std::vector<char> img(bytes);
-    put_graph(hg, p, img.data(), g->graphs, g->desc);
-    GCUDA(g, cudaMemcpyAsync(g->graphs, img.data(), bytes, cudaMemcpyHostToDevice, g->stream));
+    std::vector<char> img;
+    st = upload_graphs(g, {&hg}, {p}, {g->desc}, img);
+    if (st != QPR_OK) return st;
     qpr::GnnDev *dev = nullptr;
     st = place_group(g, g->desc, 1, &dev);
     if (st != QPR_OK) return st;
     if (backward) GCUDA(g, cudaMemsetAsync(g->loss, 0, sizeof(double), g->stream));
     enqueue_pass(g, dev, 1, hg.n, backward, true);
     *out = g->desc[0];
-    // `img` and the descriptor are free again after this
+    // the descriptor is free again after this
     GCUDA(g, cudaStreamSynchronize(g->stream));
     return QPR_OK;
 }
@@ -830,7 +908,7 @@ qpr_status qpr_gnn_train(qpr_gnn *g, int64_t count, const qpr_gnn_sample *sample
         if (!samples[i].p) return gnn_fail(g, QPR_E_ARG, "sample without target populations");
         std::string e;
         const qpr_status st = qpr::build_graph(samples[i].n, samples[i].m, samples[i].src, samples[i].dst,
-                                               samples[i].w, alpha, samples[i].omega, hg[i], e);
+                                               samples[i].w, alpha, samples[i].omega, hg[i], e, count > 4);
         if (st != QPR_OK) return gnn_fail(g, st, "sample " + std::to_string(i) + ": " + e);
     }
     // the graphs: all on the device, or a group at a time
@@ -840,25 +918,33 @@ qpr_status qpr_gnn_train(qpr_gnn *g, int64_t count, const qpr_gnn_sample *sample
     std::vector<qpr::GnnDev> graphs((size_t)count);
     std::vector<char> img;
     auto upload = [&](const std::vector<int64_t> &ids) -> qpr_status {
-        size_t bytes = 0;
-        for (int64_t i : ids) bytes += graph_bytes(hg[i]);
-        const qpr_status st = grow(g, &g->graphs, &g->graphs_cap, bytes);
-        if (st != QPR_OK) return st;
-        img.resize(bytes);
-        size_t at = 0;
+        std::vector<const qpr::HostGraph *> h;
+        std::vector<const double *> p;
+        std::vector<qpr::GnnDev *> d;
         for (int64_t i : ids) {
-            put_graph(hg[i], samples[i].p, img.data() + at, g->graphs + at, &graphs[i]);
-            at += graph_bytes(hg[i]);
+            h.push_back(&hg[i]);
+            p.push_back(samples[i].p);
+            d.push_back(&graphs[i]);
         }
-        GCUDA(g, cudaMemcpyAsync(g->graphs, img.data(), bytes, cudaMemcpyHostToDevice, g->stream));
-        GCUDA(g, cudaStreamSynchronize(g->stream));  // img is reused
-        return QPR_OK;
+        return upload_graphs(g, h, p, d, img);
     };
-    if (resident) {
-        std::vector<int64_t> all((size_t)count);
-        for (int64_t i = 0; i < count; ++i) all[i] = i;
-        const qpr_status st = upload(all);
+    for (int64_t i = 0; i < count;) {
+        // a set that does not stay: its features come back once, part by part
+        std::vector<int64_t> ids;
+        size_t bytes = 0;
+        for (; i < count && (ids.empty() || bytes + graph_bytes(hg[i]) <= kResidentBytes); ++i) {
+            ids.push_back(i);
+            bytes += graph_bytes(hg[i]);
+        }
+        const qpr_status st = upload(ids);
         if (st != QPR_OK) return st;
+        if (resident) break;
+        for (int64_t k : ids) {
+            GCUDA(g, cudaMemcpyAsync(hg[k].x.data(), graphs[k].x, hg[k].x.size() * sizeof(float), cudaMemcpyDeviceToHost,
+                                     g->stream));
+            hg[k].device_pr = false;
+        }
+        GCUDA(g, cudaStreamSynchronize(g->stream));
     }
     {
         const qpr_status st = grow_desc(g, (size_t)count);

@@ -66,6 +66,153 @@ __global__ void __launch_bounds__(kPrThreads) pagerank_step_kernel(DevOps ops, c
     if (threadIdx.x == 0) delta[blockIdx.x] = dl;
 }
 
+// Power iteration by one cluster of 8 CTAs, the iterate in every CTA's shared
+// memory (two buffers), thousands of iterations per launch. A launch per
+// iteration took 8 us at N = 922, most of it latency, with a wait for the
+// host every eighth one. What bounds an iteration here is its chain of FP64
+// instructions (40 ns each on a scheduler) and one cluster barrier, 3 us, so
+// it has as few as can be: the columns of G sum to one, so sum(pi) stays 1
+// and the teleport part (1 - alpha) (1 - pi_i) / (N - 1) needs no sum and no
+// division (rounding in the sum decays by alpha per iteration; the result is
+// normalised once). Four lanes sum a row of S (a warp one of more than kPrLong
+// entries), four warps the dangling nodes if there are any, then a thread per
+// row writes the new entry into all 8 copies through distributed shared
+// memory.
+constexpr int kPrCtas = 8;
+constexpr int kPrT = 512;
+constexpr int kPrLong = 48;
+
+__device__ __forceinline__ uint32_t pr_remote(const void *p, int cta) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n"
+                 : "=r"(r)
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(cta));
+    return r;
+}
+__device__ __forceinline__ void pr_store(uint32_t a, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;\n" ::"r"(a), "d"(v) : "memory");
+}
+__device__ __forceinline__ void pr_barrier() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+size_t pr_smem(int n) { return (size_t)(2 * n + (n + kPrCtas - 1) / kPrCtas) * sizeof(double) + n; }
+
+// jobs[blockIdx.y]. state (null: none): {iterations done, last L1 change, 1 if
+// stopped}; with it the iterate is kept in `pi` between launches (start: the
+// uniform vector when no iteration is done), and the L1 change is formed at
+// every eighth iteration and at max_iter, where the run stops (below tol, not
+// finite, or max_iter).
+__global__ void __cluster_dims__(kPrCtas, 1, 1) __launch_bounds__(kPrT, 1)
+pagerank_cluster_kernel(const PrJob *__restrict__ jobs, PrJob one, int iters, double tol, long long max_iter,
+                        double *state) {
+    extern __shared__ __align__(16) double sm[];
+    __shared__ double s_part[4], s_dang, s_delta[kPrCtas], red[32];
+    const PrJob g = jobs ? jobs[blockIdx.y] : one;
+    const int n = g.n, cta = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int per = (n + kPrCtas - 1) / kPrCtas, r0 = min(n, cta * per), rows = min(n, r0 + per) - r0;
+    double *rowsum = sm + 2 * n;
+    unsigned char *dang = reinterpret_cast<unsigned char *>(rowsum + per);
+    const bool resume = state && state[0] > 0.0;
+    int any = 0;
+    for (int i = tid; i < n; i += kPrT) {
+        sm[i] = resume ? g.pi[i] : 1.0 / n;
+        dang[i] = g.dang[i];
+        any = any || dang[i];
+    }
+    any = __syncthreads_or(any);
+    if (tid == 0) s_dang = 0.0;
+    long long it = state ? (long long)state[0] : 0;
+    const double inv_nm1 = 1.0 / (double)(n - 1), inv_n = 1.0 / (double)n;
+    const double tele = (1.0 - g.alpha) * inv_nm1;
+    __syncthreads();
+    pr_barrier();  // the cluster's CTAs run, and have read the state
+    int cur = 0;
+    bool stopped = false;
+    double delta = 0.0;
+    for (int k = 0; k < iters && !stopped; ++k) {
+        const double *pi = sm + (size_t)cur * n;
+        double *nx = sm + (size_t)(1 - cur) * n;
+        if (any && warp < 4) {
+            double D = 0.0;
+            for (int j = tid; j < n; j += 128)
+                if (dang[j]) D += pi[j];
+            D = gain64::warp_sum(D);
+            if (lane == 0) s_part[warp] = D;
+            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            if (tid == 0) s_dang = (s_part[0] + s_part[1]) + (s_part[2] + s_part[3]);
+        }
+        // quads: 8 rows of this CTA per warp and pass
+        for (int b = warp * 8; b < rows; b += (kPrT / 32) * 8) {
+            const int i = b + (lane >> 2);
+            int q0 = 0, q1 = 0;
+            if (i < rows) {
+                q0 = g.s_ptr[r0 + i];
+                q1 = g.s_ptr[r0 + i + 1];
+            }
+            const bool lng = q1 - q0 > kPrLong;
+            double s = 0.0;
+            if (!lng)
+                for (int q = q0 + (lane & 3); q < q1; q += 4) s += g.s_val[q] * pi[g.s_col[q]];
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (!lng && (lane & 3) == 0 && i < rows) rowsum[i] = s;
+            for (unsigned m = __ballot_sync(0xffffffffu, lng && (lane & 3) == 0); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const int a0 = __shfl_sync(0xffffffffu, q0, src), a1 = __shfl_sync(0xffffffffu, q1, src);
+                double t = 0.0;
+                for (int q = a0 + lane; q < a1; q += 32) t += g.s_val[q] * pi[g.s_col[q]];
+                t = gain64::warp_sum(t);
+                if (lane == 0) rowsum[b + (src >> 2)] = t;
+            }
+        }
+        __syncthreads();
+        ++it;
+        const bool check = state && (it % 8 == 0 || it >= max_iter);
+        const double D = s_dang;
+        double dl = 0.0;
+        for (int i = tid; i < rows; i += kPrT) {
+            const int gi = r0 + i;
+            const double p = pi[gi];
+            double s = rowsum[i];
+            if (any) s += (g.dangling == QPR_DANGLING_F) ? (D - (dang[gi] ? p : 0.0)) * inv_nm1 : D * inv_n;
+            const double v = g.alpha * s + tele * (1.0 - p);
+            for (int c = 0; c < kPrCtas; ++c) pr_store(pr_remote(nx + gi, c), v);
+            if (check) dl += fabs(v - p);
+        }
+        if (check) {
+            dl = block_sum(dl, red);
+            if (tid < kPrCtas) pr_store(pr_remote(s_delta + cta, tid), dl);
+        }
+        pr_barrier();
+        cur = 1 - cur;
+        if (check) {
+            delta = 0.0;
+            for (int c = 0; c < kPrCtas; ++c) delta += s_delta[c];
+            stopped = !(delta >= tol) || it >= max_iter;  // the same in every CTA
+        }
+    }
+    const double *pi = sm + (size_t)cur * n;
+    double P = 0.0;
+    if (!state || stopped) {  // normalised result
+        for (int j = tid; j < n; j += kPrT) P += pi[j];
+        P = block_sum(P, red);
+    } else {
+        P = 1.0;
+    }
+    for (int i = tid; i < rows; i += kPrT) {
+        const double v = pi[r0 + i] / P;
+        if (g.pi) g.pi[r0 + i] = v;
+        if (g.feature) g.feature[(size_t)(r0 + i) * g.stride] = (float)log((double)n * v);
+    }
+    if (state && cta == 0 && tid == 0) {
+        state[0] = (double)it;
+        state[1] = delta;
+        state[2] = stopped ? 1.0 : 0.0;
+    }
+}
+
 __global__ void uniform_kernel(double *pi, int n) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) pi[i] = 1.0 / n;
 }
@@ -146,6 +293,45 @@ cudaError_t pagerank(const DevOps &ops, double tol, int64_t max_iter, double *sc
     if (iters) *iters = it;
     if (delta_out) *delta_out = d;
     return e;
+}
+
+cudaError_t pagerank_cluster(const DevOps &ops, double tol, int64_t max_iter, double *scratch, double *pi_out_dev,
+                             int64_t *iters, double *delta_out, int64_t *launches, cudaStream_t s) {
+    const int n = ops.n;
+    PrJob job{};
+    job.n = n;
+    job.dangling = ops.dangling;
+    job.alpha = ops.alpha;
+    job.s_ptr = ops.s_ptr;
+    job.s_col = ops.s_col;
+    job.s_val = ops.s_val;
+    job.dang = ops.dang;
+    job.pi = scratch;
+    double *state = scratch + n;
+    cudaError_t e = raise_smem_limit_t(pagerank_cluster_kernel, (int)pr_smem(n));
+    if (e == cudaSuccess) e = cudaMemsetAsync(state, 0, kPrState * sizeof(double), s);
+    double h[kPrState] = {0.0, INFINITY, 0.0, 0.0};
+    *launches = 0;
+    while (e == cudaSuccess && h[2] == 0.0) {
+        pagerank_cluster_kernel<<<kPrCtas, kPrT, pr_smem(n), s>>>(nullptr, job, 4096, tol, (long long)max_iter, state);
+        ++*launches;
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(h, state, sizeof(h), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(pi_out_dev, scratch, n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    if (iters) *iters = (int64_t)h[0];
+    if (delta_out) *delta_out = h[1];
+    return e;
+}
+
+cudaError_t pagerank_jobs(const PrJob *jobs, int count, int max_n, int iters, cudaStream_t s) {
+    cudaError_t e = raise_smem_limit_t(pagerank_cluster_kernel, (int)pr_smem(max_n));
+    if (e != cudaSuccess) return e;
+    for (int at = 0; at < count; at += 32768)
+        pagerank_cluster_kernel<<<dim3(kPrCtas, std::min(count - at, 32768)), kPrT, pr_smem(max_n), s>>>(
+            jobs + at, PrJob{}, iters, 0.0, 0, nullptr);
+    return cudaGetLastError();
 }
 
 cudaError_t hub_classes(const double *p, int n, double c, int *classes_dev, unsigned long long *counts_dev,

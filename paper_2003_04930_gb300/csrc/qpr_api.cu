@@ -1,6 +1,7 @@
 // Host runtime and C ABI of the solver: argument validation, operator
 // assembly (Supplementary Note 1), the RK4 driver with CUDA-graph capture and
 // device-side stop decision, and the host/device pointer handling.
+#include <limits.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -64,6 +65,7 @@ struct qpr_ctx {
     int4 *d_epi_pairs = nullptr, *d_pairs64 = nullptr;
     Ctl *d_ctl = nullptr;
     double *d_io = nullptr;     // staging for host density matrices (interleaved)
+    double *d_pr = nullptr;     // PageRank: the iterate and its state (kPrScratch)
     double *d_p = nullptr;      // populations staging
     float *d_rkf = nullptr;     // RKF45: D1, Dlo1, acc, Flo (2 planes each), the two compact diagonals
     cudaGraphExec_t graph_rkf = nullptr;  // RKF45: refresh + ref_refresh attempts
@@ -571,7 +573,7 @@ void row_segments(const HostOps &h, int np, int len, std::vector<int> &rowseg, s
 // out-degrees, CSR of H (Eq. S6) and of S (column-normalised adjacency
 // restricted to columns with out-links), dangling flags.
 qpr_status assemble_host(int64_t n, int64_t m, const int64_t *src, const int64_t *dst, const double *w, int h_diag,
-                         HostOps &out, std::string &err) {
+                         HostOps &out, std::string &err, bool with_h) {
     out.n = n;
     for (int64_t e = 0; e < m; ++e) {
         const double we = w ? w[e] : 1.0;
@@ -581,62 +583,76 @@ qpr_status assemble_host(int64_t n, int64_t m, const int64_t *src, const int64_t
             { err = "edge " + std::to_string(e) + " has a negative or non-finite weight"; return QPR_E_GRAPH; }
     }
 
-    // ---- adjacency: A_ij = w for the link j -> i; duplicates sum ----
-    struct Ent { int64_t i, j; double a; };
-    std::vector<Ent> ents;
-    ents.reserve((size_t)m);
-    for (int64_t e = 0; e < m; ++e) {
-        const double we = w ? w[e] : 1.0;
-        if (src[e] == dst[e] || we == 0.0) continue;
-        ents.push_back({dst[e], src[e], we});
-    }
-    std::stable_sort(ents.begin(), ents.end(), [](const Ent &x, const Ent &y) {
-        return x.i != y.i ? x.i < y.i : x.j < y.j;
-    });
-    std::vector<Ent> A;
-    for (const Ent &x : ents) {
-        if (!A.empty() && A.back().i == x.i && A.back().j == x.j) A.back().a += x.a;
-        else A.push_back(x);
+    // ---- adjacency in CSR: A_ij = w for the link j -> i; duplicates sum ----
+    // (bucketed by row, each row sorted by column; equal columns keep edge order)
+    std::vector<int64_t> aptr(n + 1, 0);
+    for (int64_t e = 0; e < m; ++e)
+        if (src[e] != dst[e] && (!w || w[e] != 0.0)) ++aptr[dst[e] + 1];
+    for (int64_t i = 0; i < n; ++i) aptr[i + 1] += aptr[i];
+    struct Ent { int j; double a; };
+    std::vector<Ent> A((size_t)aptr[n]);
+    {
+        std::vector<int64_t> at(aptr.begin(), aptr.end() - 1);
+        for (int64_t e = 0; e < m; ++e)
+            if (src[e] != dst[e] && (!w || w[e] != 0.0)) A[at[dst[e]]++] = {(int)src[e], w ? w[e] : 1.0};
+        size_t q = 0;
+        for (int64_t i = 0; i < n; ++i) {
+            const size_t q0 = (size_t)aptr[i], q1 = (size_t)aptr[i + 1], first = q;
+            std::stable_sort(A.begin() + q0, A.begin() + q1, [](const Ent &x, const Ent &y) { return x.j < y.j; });
+            for (size_t k = q0; k < q1; ++k) {
+                if (q > first && A[q - 1].j == A[k].j) A[q - 1].a += A[k].a;
+                else A[q++] = A[k];
+            }
+            aptr[i] = (int64_t)first;
+        }
+        aptr[n] = (int64_t)q;
+        A.resize(q);
     }
     std::vector<double> &outdeg = out.outdeg;
     outdeg.assign(n, 0.0);
     for (const Ent &x : A) outdeg[x.j] += x.a;
 
-    // ---- H (Eq. S6): H_ij = -max(A_ij, A_ji) off the diagonal ----
-    std::vector<Ent> Hs;
-    Hs.reserve(A.size() * 2);
-    for (const Ent &x : A) {
-        Hs.push_back({x.i, x.j, x.a});
-        Hs.push_back({x.j, x.i, x.a});
-    }
-    std::sort(Hs.begin(), Hs.end(), [](const Ent &x, const Ent &y) {
-        return x.i != y.i ? x.i < y.i : x.j < y.j;
-    });
-    std::vector<Ent> Hu;  // unique (i, j) with -max
-    for (const Ent &x : Hs) {
-        if (!Hu.empty() && Hu.back().i == x.i && Hu.back().j == x.j) Hu.back().a = std::max(Hu.back().a, x.a);
-        else Hu.push_back(x);
-    }
-    std::vector<int64_t> &hptr = out.hptr;
-    std::vector<int> &hcol = out.hcol;
-    std::vector<double> &hval = out.hval;
-    hptr.assign(n + 1, 0);
-    {
-        size_t q = 0;
+    // ---- H (Eq. S6): H_ij = -max(A_ij, A_ji) off the diagonal: the union of
+    // the rows of A and of its transpose ----
+    if (with_h) {
+        std::vector<int64_t> tptr(n + 1, 0);
+        for (const Ent &x : A) ++tptr[x.j + 1];
+        for (int64_t i = 0; i < n; ++i) tptr[i + 1] += tptr[i];
+        std::vector<Ent> T(A.size());
+        {
+            std::vector<int64_t> at(tptr.begin(), tptr.end() - 1);
+            for (int64_t i = 0; i < n; ++i)
+                for (int64_t q = aptr[i]; q < aptr[i + 1]; ++q) T[at[A[q].j]++] = {(int)i, A[q].a};
+        }
+        std::vector<int64_t> &hptr = out.hptr;
+        std::vector<int> &hcol = out.hcol;
+        std::vector<double> &hval = out.hval;
+        hptr.assign(n + 1, 0);
+        hcol.reserve(2 * A.size());
+        hval.reserve(2 * A.size());
         for (int64_t i = 0; i < n; ++i) {
             hptr[i] = (int64_t)hcol.size();
-            bool diag_done = false;
             const double hd = (h_diag == QPR_HDIAG_NEG_OUTDEG) ? -outdeg[i] : 0.0;
-            while (q < Hu.size() && Hu[q].i == i) {
-                if (!diag_done && Hu[q].j > i) {
-                    if (hd != 0.0) { hcol.push_back((int)i); hval.push_back(hd); }
+            bool diag_done = hd == 0.0;
+            int64_t qa = aptr[i], qt = tptr[i];
+            while (qa < aptr[i + 1] || qt < tptr[i + 1]) {
+                const int ja = qa < aptr[i + 1] ? A[qa].j : INT_MAX, jt = qt < tptr[i + 1] ? T[qt].j : INT_MAX;
+                const int j = std::min(ja, jt);
+                double v = 0.0;
+                if (ja == j) v = A[qa++].a;
+                if (jt == j) v = std::max(v, T[qt++].a);
+                if (!diag_done && j > i) {
+                    hcol.push_back((int)i);
+                    hval.push_back(hd);
                     diag_done = true;
                 }
-                hcol.push_back((int)Hu[q].j);
-                hval.push_back(-Hu[q].a);
-                ++q;
+                hcol.push_back(j);
+                hval.push_back(-v);
             }
-            if (!diag_done && hd != 0.0) { hcol.push_back((int)i); hval.push_back(hd); }
+            if (!diag_done) {
+                hcol.push_back((int)i);
+                hval.push_back(hd);
+            }
         }
         hptr[n] = (int64_t)hcol.size();
     }
@@ -647,17 +663,10 @@ qpr_status assemble_host(int64_t n, int64_t m, const int64_t *src, const int64_t
     sptr.assign(n + 1, 0);
     scol.reserve(A.size());
     sval.reserve(A.size());
-    {
-        size_t q = 0;
-        for (int64_t i = 0; i < n; ++i) {
-            sptr[i] = (int)scol.size();
-            while (q < A.size() && A[q].i == i) {
-                scol.push_back((int)A[q].j);
-                sval.push_back(A[q].a / outdeg[A[q].j]);
-                ++q;
-            }
-        }
-        sptr[n] = (int)scol.size();
+    for (int64_t i = 0; i <= n; ++i) sptr[i] = (int)aptr[i];
+    for (const Ent &x : A) {
+        scol.push_back(x.j);
+        sval.push_back(x.a / outdeg[x.j]);
     }
     std::vector<unsigned char> &dang = out.dang;
     dang.assign(n, 0);
@@ -786,6 +795,7 @@ void qpr_destroy(qpr_ctx *ctx) {
     cudaFree(ctx->d_ctl);
     cudaFree(ctx->d_io);
     cudaFree(ctx->d_p);
+    cudaFree(ctx->d_pr);
     if (ctx->h_ctl) cudaFreeHost(ctx->h_ctl);
     if (ctx->ev) cudaEventDestroy(ctx->ev);
     if (ctx->stream) cudaStreamDestroy(ctx->stream);
@@ -1077,6 +1087,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     CREATE_CUDA(cudaMemset(ctx->d_ctl, 0, sizeof(Ctl)));
     CREATE_CUDA(cudaMalloc(&ctx->d_io, (size_t)n * n * 2 * sizeof(double)));
     CREATE_CUDA(cudaMalloc(&ctx->d_p, n * sizeof(double)));
+    if (n <= qpr::kPrClusterMaxN) CREATE_CUDA(cudaMalloc(&ctx->d_pr, ((size_t)n + qpr::kPrState) * sizeof(double)));
     CREATE_CUDA(cudaMallocHost(&ctx->h_ctl, sizeof(Ctl)));
     CREATE_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
     CREATE_CUDA(cudaEventCreateWithFlags(&ctx->ev, cudaEventDisableTiming));
@@ -1624,13 +1635,15 @@ qpr_status qpr_pagerank(qpr_ctx *ctx, double tol, int64_t max_iter, double *pi, 
     if (!pi) return fail(ctx, QPR_E_ARG, "pi is NULL");
     if (!(tol > 0.0) || max_iter < 1) return fail(ctx, QPR_E_ARG, "tol must be positive and max_iter >= 1");
     const int64_t n = ctx->n;
-    // scratch: the host staging buffer (2 n^2 doubles >= 2 n + grid for n >= 2)
-    if ((size_t)2 * n * n < (size_t)(2 * n + qpr::pagerank_grid((int)n)))
-        return fail(ctx, QPR_E_ARG, "n too small for the staging buffer");
-    int64_t it = 0;
+    int64_t it = 0, launches = 0;
     double delta = 0.0;
-    QPR_CUDA(ctx, qpr::pagerank(ctx->ops, tol, max_iter, ctx->d_io, ctx->d_p, &it, &delta, ctx->stream));
-    ctx->launches += 2 + it;
+    if (n <= qpr::kPrClusterMaxN) {
+        QPR_CUDA(ctx, qpr::pagerank_cluster(ctx->ops, tol, max_iter, ctx->d_pr, ctx->d_p, &it, &delta, &launches, ctx->stream));
+    } else {
+        QPR_CUDA(ctx, qpr::pagerank(ctx->ops, tol, max_iter, ctx->d_io, ctx->d_p, &it, &delta, ctx->stream));
+        launches = 2 + it;
+    }
+    ctx->launches += launches;
     if (is_device_ptr(pi)) {
         QPR_CUDA(ctx, cudaMemcpyAsync(pi, ctx->d_p, n * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     } else {

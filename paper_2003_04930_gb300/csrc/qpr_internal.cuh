@@ -388,6 +388,25 @@ int pagerank_grid(int n);
 // 2 n + pagerank_grid(n) doubles. Synchronises the stream.
 cudaError_t pagerank(const DevOps &ops, double tol, int64_t max_iter, double *scratch, double *pi_out_dev,
                      int64_t *iters, double *delta_out, cudaStream_t s);
+// The same for n <= kPrClusterMaxN in one cluster per graph, up to a few
+// thousand iterations per launch. scratch: n + kPrState doubles.
+constexpr int kPrClusterMaxN = 8192;
+constexpr int kPrState = 4;
+cudaError_t pagerank_cluster(const DevOps &ops, double tol, int64_t max_iter, double *scratch, double *pi_out_dev,
+                             int64_t *iters, double *delta_out, int64_t *launches, cudaStream_t s);
+// A fixed number of power iterations for `count` graphs of at most max_n <=
+// kPrClusterMaxN nodes (jobs in device memory), from the uniform vector.
+struct PrJob {
+    int n, dangling;
+    double alpha;
+    const int *s_ptr, *s_col;
+    const double *s_val;
+    const unsigned char *dang;
+    double *pi;       // n: the normalised vector (may be null)
+    float *feature;   // (float)log(n pi_i) at feature[i * stride] (may be null)
+    int stride;
+};
+cudaError_t pagerank_jobs(const PrJob *jobs, int count, int max_n, int iters, cudaStream_t s);
 // classes_dev[i] in {0, 1, 2} (rest, secondary hub, main hub) of the
 // probabilities p (device, n doubles) with threshold factor c; counts_dev
 // (3 values) receives the class sizes.
@@ -416,7 +435,7 @@ struct HostOps {
     std::vector<unsigned char> dang;
 };
 qpr_status assemble_host(int64_t n, int64_t m, const int64_t *src, const int64_t *dst, const double *w, int h_diag,
-                         HostOps &out, std::string &err);
+                         HostOps &out, std::string &err, bool with_h = true);
 // Segments of at most `len` nonzeros of every row of the CSR of H, for np
 // rows (rowseg: np + 1 entries, seg: {q0, q1}).
 void row_segments(const HostOps &h, int np, int len, std::vector<int> &rowseg, std::vector<int2> &seg);
