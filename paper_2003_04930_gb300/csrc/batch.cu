@@ -135,75 +135,108 @@ __global__ void __launch_bounds__(kStageNT) b_stage_mixed_kernel(const BatchGrap
 // Column-block form: the SpMM over (problem, J, split) items. The split's
 // entries and bundles (two bulk copies) and the column block (3-D tensor
 // loads through the problem's own tensor map, kept in device memory) land
-// on one mbarrier while the CTA forms its share of the problem's gain; the
+// on mbarriers while the CTA forms its share of the problem's gain; the
 // arithmetic is the single-problem form's (warp_bundles, cta_gain), so the
 // results are bitwise the same. Registers are capped for two resident CTAs
 // per SM, so that the small size classes (less shared memory) overlap one
 // CTA's staging with another's products.
+//
+// A batch of small problems is latency from end to end (12 problems of N <=
+// 492: 27 us a stage, for arithmetic worth half of it), so both kernels of a
+// stage are launched with programmatic dependent launch: this one fetches its
+// first item's descriptor, entries and bundles, which no kernel writes, before
+// it waits; the epilogue its first item's operands, which are complete once
+// every CTA of this kernel has passed its own wait.
 template <int STAGE>
 __global__ void __launch_bounds__(cols::kANT, 2) b_cols_spmm_kernel(const BatchGraph *gs, const Ctl *ctls,
                                                                  const int4 *items, int nitems) {
     extern __shared__ __align__(128) uint8_t dyn_smem[];
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
-    __shared__ __align__(8) uint64_t bar;
+    __shared__ __align__(8) uint64_t bar_csr, bar_d;
     if (threadIdx.x == 0) {
-        tma::mbar_init(&bar, 1);
+        tma::mbar_init(&bar_csr, 1);
+        tma::mbar_init(&bar_d, 1);
         tma::mbar_init_fence();
     }
-    uint32_t phase = 0;
+    // 128-byte aligned for the tensor loads (the plan's size leaves the slack)
+    const uint32_t s0 = tma::smem_u32(dyn_smem);
+    uint8_t *base = dyn_smem + (((s0 + 127) & ~127u) - s0);
+    float *sD = reinterpret_cast<float *>(base);
+    uint32_t phase_csr = 0, phase_d = 0;
+    bool first = true;
     int4 tn = blockIdx.x < nitems ? items[blockIdx.x] : make_int4(0, 0, 0, 0);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 t = tn;
         if (it + (int)gridDim.x < nitems) tn = items[it + gridDim.x];  // the next item, in flight meanwhile
-        if (!load_graph_done(gs, ctls, t.x, sg, &s_flag)) {
+        int done = 0;
+        if (first) load_graph(gs, t.x, sg);
+        else done = load_graph_done(gs, ctls, t.x, sg, &s_flag);
+        if (!done) {
             const DevOps &ops = sg.ops;
             const int J = t.y, r = t.z, np = ops.np;
-            // 128-byte aligned for the tensor loads (the plan's size leaves the slack)
-            const uint32_t s0 = tma::smem_u32(dyn_smem);
-            uint8_t *base = dyn_smem + (((s0 + 127) & ~127u) - s0);
-            float *sD = reinterpret_cast<float *>(base);
             int2 *sKH = reinterpret_cast<int2 *>(base + (size_t)np * cols::kRowFloats * 4);
             int4 *sP = reinterpret_cast<int4 *>(base + ops.col_p_off);
             const int q_base = ops.col_q[2 * r], q_end = ops.col_q[2 * r + 1];
             const int p_base = ops.col_sb[r], p_end = ops.col_sb[r + 1];
-            if (threadIdx.x < 32) {
+            if (threadIdx.x == 0) {
                 // the previous item's reads of these buffers came through the generic proxy
                 asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 const uint32_t kh_bytes = (uint32_t)((q_end - q_base) * 8);
                 const uint32_t p_bytes = (uint32_t)((p_end - p_base) * 16 * cols::kBundleInt4);
-                const uint32_t d_bytes = (uint32_t)np * cols::kRowFloats * 4;
+                tma::mbar_expect_tx(&bar_csr, kh_bytes + p_bytes);
+                if (kh_bytes) tma::load_bulk(sKH, ops.col_kh + q_base, kh_bytes, &bar_csr);
+                if (p_bytes)
+                    tma::load_bulk(sP, ops.col_pieces + cols::kBundleInt4 * (size_t)p_base, p_bytes, &bar_csr);
+            }
+            if (first) {
+                tma::grid_dependency_wait();
+                tma::launch_dependents();
+                if (threadIdx.x == 0) s_flag = *(volatile const int *)&ctls[t.x].done;
+                __syncthreads();
+                done = s_flag;
+            }
+            bool ok = true;
+            if (!done) {
                 if (threadIdx.x == 0) {
-                    tma::mbar_expect_tx(&bar, kh_bytes + p_bytes + d_bytes);
-                    if (kh_bytes) tma::load_bulk(sKH, ops.col_kh + q_base, kh_bytes, &bar);
-                    if (p_bytes)
-                        tma::load_bulk(sP, ops.col_pieces + cols::kBundleInt4 * (size_t)p_base, p_bytes, &bar);
+                    tma::mbar_expect_tx(&bar_d, (uint32_t)np * cols::kRowFloats * 4);
                     // the stage input's map: D (stage 1), da (stages 2 and 4), db (stage 3)
                     const CUtensorMap *tm = &sg.dmaps->d[STAGE == 1 ? 0 : (STAGE == 3 ? 2 : 1)];
                     for (int b = 0; b < np; b += cols::kBoxRows)
-                        tma::load_3d(sD + (size_t)b * cols::kRowFloats, tm, &bar, J * cols::kCW, 0, b);
+                        tma::load_3d(sD + (size_t)b * cols::kRowFloats, tm, &bar_d, J * cols::kCW, 0, b);
                 }
+                const int ncb = np / cols::kCW;
+                // the step's stop decision, by one unit of the problem's stage-2
+                // grid (as a ticket in the stage-1 epilogue it took 6 us); the
+                // other units' products are scratch then
+                if (STAGE == 2 && J == ncb - 1 && r == ops.col_splits - 1)
+                    cols::stage1_decision(sg.mw, sg.mw.npairs, *(volatile long long *)&sg.mw.ctl->step, true);
+                cols::cta_gain(ops, sg.mw, r * ncb + J, ncb * ops.col_splits,
+                               reinterpret_cast<float *>(base + ops.col_sp_off));
+                ok = tma::mbar_wait(&bar_d, phase_d & 1);
+                ++phase_d;
             }
-            const int ncb = np / cols::kCW;
-            cols::cta_gain(ops, sg.mw, r * ncb + J, ncb * ops.col_splits,
-                           reinterpret_cast<float *>(base + ops.col_sp_off));
-            const bool ok = tma::mbar_wait(&bar, phase & 1);
-            ++phase;
+            ok = tma::mbar_wait(&bar_csr, phase_csr & 1) && ok;
+            ++phase_csr;
             if (__syncthreads_or(!ok)) {
                 if (threadIdx.x == 0) atomicExch(&sg.mw.ctl->err_timeout, 1);
-                tma::mbar_wait(&bar, (phase - 1) & 1);
+                tma::mbar_wait(&bar_csr, (phase_csr - 1) & 1);
+                if (!done) tma::mbar_wait(&bar_d, (phase_d - 1) & 1);
                 return;
             }
-            const int warp = threadIdx.x >> 5;
-            float *parts = reinterpret_cast<float *>(base + ops.col_part_off);
-            cols::warp_bundles(sD, sKH, sP, p_base, ops.col_wb[r * cols::kAWarps + warp],
-                               ops.col_wb[r * cols::kAWarps + warp + 1], J, np, sg.mw.X, parts);
-            const int cb0 = ops.col_cutb[r], cb1 = ops.col_cutb[r + 1];
-            if (cb1 > cb0) {
-                __syncthreads();
-                cols::combine_cuts(ops.col_cut + cb0, cb1 - cb0, parts, J, np, sg.mw.X);
+            if (!done) {
+                const int warp = threadIdx.x >> 5;
+                float *parts = reinterpret_cast<float *>(base + ops.col_part_off);
+                cols::warp_bundles(sD, sKH, sP, p_base, ops.col_wb[r * cols::kAWarps + warp],
+                                   ops.col_wb[r * cols::kAWarps + warp + 1], J, np, sg.mw.X, parts);
+                const int cb0 = ops.col_cutb[r], cb1 = ops.col_cutb[r + 1];
+                if (cb1 > cb0) {
+                    __syncthreads();
+                    cols::combine_cuts(ops.col_cut + cb0, cb1 - cb0, parts, J, np, sg.mw.X);
+                }
             }
         }
+        first = false;
         __syncthreads();
     }
 }
@@ -218,12 +251,30 @@ __global__ void __launch_bounds__(cols::kENT, 3) b_cols_epi_kernel(const BatchGr
     __shared__ float sg32[mixed::TS];
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    bool first = true;
     int4 tn = blockIdx.x < nitems ? items[blockIdx.x] : make_int4(0, 0, 0, 0);
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 t = tn;
         if (it + (int)gridDim.x < nitems) tn = items[it + gridDim.x];  // the next item, in flight meanwhile
-        if (!load_graph_done(gs, ctls, t.x, sg, &s_flag))
-            cols::epilogue_pair<STAGE>(sg.ops, sg.mw, t.y, t.z, t.w, t.w == 0, sg.mw.npairs, sX1, sX2, sg32, sO);
+        mixed::EpiIn<STAGE, cols::kENT> in;
+        int done;
+        if (first) {
+            // the operands before the wait, the stop flag (set by a stage-2 product) after it
+            load_graph(gs, t.x, sg);
+            mixed::epi_load<STAGE, cols::kENT>(sg.ops, sg.mw, t.y, t.z, in);
+            tma::grid_dependency_wait();
+            tma::launch_dependents();
+            if (threadIdx.x == 0) s_flag = *(volatile const int *)&ctls[t.x].done;
+            __syncthreads();
+            done = s_flag;
+        } else {
+            done = load_graph_done(gs, ctls, t.x, sg, &s_flag);
+            if (!done) mixed::epi_load<STAGE, cols::kENT>(sg.ops, sg.mw, t.y, t.z, in);
+        }
+        if (!done)
+            cols::epilogue_pair_in<STAGE>(sg.ops, sg.mw, t.y, t.z, t.w, t.w == 0, sg.mw.npairs, sX1, sX2, sg32,
+                                                 sO, in);
+        first = false;
         __syncthreads();
     }
 }
@@ -287,7 +338,23 @@ void launch_refresh(const BatchGraph *gs, const Lists &L, int max_np, cudaStream
     b_sparse64_kernel<<<std::min(L.nitems, 152 * 3), sparse64::NTHREADS, sparse64::SMEM_BYTES, s>>>(gs, L.items,
                                                                                                      L.nitems, due);
     b_post_kernel<<<eg, 256, 0, s>>>(gs, L.act, due);
-    launches += 5;
+    launches += 4;
+}
+
+// Programmatic dependent launch on the stream.
+template <typename K, typename... A>
+void launch_dep(K kernel, int grid, int block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
 template <int STAGE>
@@ -295,12 +362,14 @@ void launch_stage_b(const BatchGraph *gs, const Ctl *ctls, const Lists &L, cudaS
     bool any = false;
     for (int c = 0; c < kClasses; ++c)
         if (L.na[c]) {
-            b_cols_spmm_kernel<STAGE><<<L.grid_a[c], cols::kANT, L.smem_a[c], s>>>(gs, ctls, L.items_a[c], L.na[c]);
+            launch_dep(b_cols_spmm_kernel<STAGE>, L.grid_a[c], cols::kANT, (size_t)L.smem_a[c], s, gs, ctls,
+                       (const int4 *)L.items_a[c], L.na[c]);
             launches += 1;
             any = true;
         }
     if (any) {
-        b_cols_epi_kernel<STAGE><<<std::min(L.nb, 152 * 3), cols::kENT, 0, s>>>(gs, ctls, L.items_b, L.nb);
+        launch_dep(b_cols_epi_kernel<STAGE>, std::min(L.nb, 152 * 3), cols::kENT, 0, s, gs, ctls,
+                   (const int4 *)L.items_b, L.nb);
         launches += 1;
     }
     if (L.nt) {
@@ -483,9 +552,25 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     size_t nkh = 0, nci = 0, npc = 0, nxc = 0, na_max = 0;
     int smem_a = 0;
     int smem_class[qpr::kClasses] = {};
+    // Row splits: one where it fits and the batch fills the SMs with many
+    // problems; in a small batch, as many as bring a unit's entries down to an
+    // even share, with no more units than two CTAs per SM take at once (a
+    // row's sum does not depend on the split). 12 problems of N <= 492: 119 us a
+    // step with 407 units (two rounds on some SMs), 96 with 304.
+    double share = 512.0;
+    {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        for (; share < 1e9; share *= 1.1) {
+            int64_t units = 0;
+            for (size_t g = 0; g < G; ++g)
+                units += (np[g] / qpr::cols::kCW) * (int64_t)std::max(1.0, std::min(8.0, ceil((double)H[g].hval.size() / share)));
+            if (units <= 2 * (int64_t)std::max(sms, 1)) break;
+        }
+    }
     for (size_t g = 0; g < G; ++g) {
-        // one split where it fits: the batch fills the SMs with many problems
-        if (o.sparse_form == QPR_SPARSE_FORM_TILES || !qpr::plan_columns(H[g], np[g], dev, plans[g], 1)) {
+        const int splits = std::min(8, std::max(1, (int)ceil((double)H[g].hval.size() / share)));
+        if (o.sparse_form == QPR_SPARSE_FORM_TILES || !qpr::plan_columns(H[g], np[g], dev, plans[g], splits)) {
             if (o.sparse_form == QPR_SPARSE_FORM_COLUMNS || o.sparse_form == QPR_SPARSE_FORM_COLUMNS_PERSISTENT)
                 return err(QPR_E_ARG, "problem " + std::to_string(g) +
                                           ": sparse_form COLUMNS does not fit one CTA's shared memory");

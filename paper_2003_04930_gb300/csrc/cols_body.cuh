@@ -372,9 +372,9 @@ __device__ __forceinline__ void cta_gain(const DevOps &ops, const MixedWork &w, 
 // estimate to ctl and, when the run stops here, sets done so that the later
 // kernels of the step return at once. A step whose exact residual a refresh
 // already decided is not decided again. Returns the status. Callers: the
-// first gain CTA of the stage-2 SpMM grid (single-problem column forms, RK4
-// and RKF45), every CTA of the persistent form's stage 2, and the last CTA
-// of a problem's stage-1 epilogue in the batched solver.
+// first gain CTA of the stage-2 SpMM grid (single-problem column and dense
+// forms, RK4 and RKF45), every CTA of the persistent form's stage 2, and one
+// unit of a problem's stage-2 SpMM in the batched solver.
 __device__ __forceinline__ int stage1_decision(const MixedWork &w, int nparts, long long step, bool record) {
     __shared__ float red[32];
     __shared__ int s_status;
@@ -404,25 +404,8 @@ __device__ __forceinline__ int stage1_decision(const MixedWork &w, int nparts, l
     return s_status;
 }
 
-// The last CTA to finish a stage-1 epilogue (a ticket in the control block;
-// release/acquire through fences) takes the stop decision.
-__device__ __forceinline__ void stage1_last_decides(const MixedWork &w, int nparts) {
-    __shared__ int s_last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = (atomicAdd(&w.ctl->ticket, 1) == nparts - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (threadIdx.x == 0) w.ctl->ticket = 0;
-    stage1_decision(w, nparts, *(volatile long long *)&w.ctl->step, true);
-}
-
 // Epilogue of tile pair (I, J) from X (global, written by the SpMM kernel)
-// and the gain w.g (both read from L2: other CTAs wrote them); stage 1 ends
-// with the ticket of the stop decision (TICKET),
-// stage 4 advances the step counter (first pair). kENT threads. Shared
+// and the gain w.g (both read from L2: other CTAs wrote them); stage 4 advances the step counter (first pair). kENT threads. Shared
 // memory: sX1, sX2 (TS * LDX floats each), sg (TS), sO (4 * TS * LDO).
 // The X tiles of pair (I, J) into sX1 (X_IJ) and sX2 (X_JI, off-diagonal
 // pairs), and the gain of a diagonal pair into sg; no barrier at the end.
@@ -451,32 +434,31 @@ __device__ __forceinline__ void epilogue_load_x(const DevOps &ops, const MixedWo
 
 // The epilogue of pair (I, J) once its X tiles and gain are in shared memory
 // (after a barrier).
-template <int STAGE, bool TICKET = true, bool SPLIT = false>
+template <int STAGE, bool SPLIT = false>
 __device__ __forceinline__ void epilogue_pair_staged(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
                                                      bool first, int nparts, const float *sX1, const float *sX2,
                                                      const float *sg, float *sO, const mixed::EpiIn<STAGE, kENT> &in) {
     mixed::tile_epilogue_in<STAGE, kENT, SPLIT>(ops, w, I, J, pidx, sX1, sX2, sg, sO, in);
-    if (STAGE == 1 && TICKET) stage1_last_decides(w, nparts);
     if (STAGE == 4 && first && threadIdx.x == 0) w.ctl->step += 1;
 }
 
-template <int STAGE, bool TICKET = true>
+template <int STAGE>
 __device__ __forceinline__ void epilogue_pair_in(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
                                                  bool first, int nparts, float *sX1, float *sX2, float *sg, float *sO,
                                                  const mixed::EpiIn<STAGE, kENT> &in) {
     epilogue_load_x(ops, w, I, J, sX1, sX2, sg);
     __syncthreads();
-    epilogue_pair_staged<STAGE, TICKET>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
+    epilogue_pair_staged<STAGE>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
 }
 
 // The same with the elementwise operands loaded first, so that their loads
 // and the X tiles' are in flight together.
-template <int STAGE, bool TICKET = true>
+template <int STAGE>
 __device__ __forceinline__ void epilogue_pair(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
                                               bool first, int nparts, float *sX1, float *sX2, float *sg, float *sO) {
     mixed::EpiIn<STAGE, kENT> in;
     mixed::epi_load<STAGE, kENT>(ops, w, I, J, in);
-    epilogue_pair_in<STAGE, TICKET>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
+    epilogue_pair_in<STAGE>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
 }
 
 }  // namespace cols
