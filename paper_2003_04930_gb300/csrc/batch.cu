@@ -78,18 +78,30 @@ __device__ __forceinline__ int skip_refresh(const BatchGraph &sg, int g, const u
     return due && !due[g];
 }
 
-__global__ void __launch_bounds__(256) b_trace_kernel(const BatchGraph *gs, const int *act, const uint8_t *due) {
+// The lists a captured block runs over change as problems stop; their lengths
+// are read from device memory, so one capture serves the whole solve (with a
+// capture at every change 12 problems of N <= 492 took 246 ms, 227 so and with
+// the spectra formed on the device).
+struct Counts {
+    int act, items, b, t;  // active problems, all pairs, column-form pairs, tile-form pairs
+    int a[2];              // SpMM units per size class
+};
+
+__global__ void __launch_bounds__(256) b_trace_kernel(const BatchGraph *gs, const int *act, const Counts *cn,
+                                                      const uint8_t *due) {
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    if ((int)blockIdx.x >= cn->act) return;
     load_graph(gs, act[blockIdx.x], sg);
     if (skip_refresh(sg, act[blockIdx.x], due, &s_flag)) return;
     mixed::refresh_trace_body(sg.ops, sg.mw);
 }
 
-__global__ void __launch_bounds__(256) b_normalize_kernel(const BatchGraph *gs, const int *act,
+__global__ void __launch_bounds__(256) b_normalize_kernel(const BatchGraph *gs, const int *act, const Counts *cn,
                                                           const uint8_t *due) {
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    if ((int)blockIdx.y >= cn->act) return;
     load_graph(gs, act[blockIdx.y], sg);
     if (skip_refresh(sg, act[blockIdx.y], due, &s_flag)) return;
     mixed::refresh_normalize_body(sg.ops, sg.mw, blockIdx.x * (size_t)blockDim.x + threadIdx.x,
@@ -97,10 +109,11 @@ __global__ void __launch_bounds__(256) b_normalize_kernel(const BatchGraph *gs, 
 }
 
 __global__ void __launch_bounds__(sparse64::NTHREADS)
-b_sparse64_kernel(const BatchGraph *gs, const int4 *items, int nitems, const uint8_t *due) {
+b_sparse64_kernel(const BatchGraph *gs, const int4 *items, const Counts *cn, const uint8_t *due) {
     extern __shared__ __align__(16) double smem[];
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    const int nitems = cn->items;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 t = items[it];
         load_graph(gs, t.x, sg);
@@ -109,9 +122,11 @@ b_sparse64_kernel(const BatchGraph *gs, const int4 *items, int nitems, const uin
     }
 }
 
-__global__ void __launch_bounds__(256) b_post_kernel(const BatchGraph *gs, const int *act, const uint8_t *due) {
+__global__ void __launch_bounds__(256) b_post_kernel(const BatchGraph *gs, const int *act, const Counts *cn,
+                                                     const uint8_t *due) {
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    if ((int)blockIdx.y >= cn->act) return;
     load_graph(gs, act[blockIdx.y], sg);
     if (skip_refresh(sg, act[blockIdx.y], due, &s_flag)) return;
     mixed::refresh_post_body(sg.ops, sg.mw, blockIdx.x * (size_t)blockDim.x + threadIdx.x,
@@ -119,10 +134,11 @@ __global__ void __launch_bounds__(256) b_post_kernel(const BatchGraph *gs, const
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(kStageNT) b_stage_mixed_kernel(const BatchGraph *gs, const int4 *items, int nitems) {
+__global__ void __launch_bounds__(kStageNT) b_stage_mixed_kernel(const BatchGraph *gs, const int4 *items, const Counts *cn) {
     extern __shared__ __align__(16) uint8_t tile_smem[];
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
+    const int nitems = cn->t;
     for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
         const int4 t = items[it];
         load_graph(gs, t.x, sg);
@@ -149,7 +165,12 @@ __global__ void __launch_bounds__(kStageNT) b_stage_mixed_kernel(const BatchGrap
 // every CTA of this kernel has passed its own wait.
 template <int STAGE>
 __global__ void __launch_bounds__(cols::kANT, 2) b_cols_spmm_kernel(const BatchGraph *gs, const Ctl *ctls,
-                                                                 const int4 *items, int nitems) {
+                                                                 const int4 *items, const Counts *cn, int cls) {
+    const int nitems = cn->a[cls];
+    if ((int)blockIdx.x >= nitems) {
+        tma::grid_dependency_wait();  // a launch without items still ends after the ones before it
+        return;
+    }
     extern __shared__ __align__(128) uint8_t dyn_smem[];
     __shared__ BatchGraph sg;
     __shared__ int s_flag;
@@ -244,7 +265,12 @@ __global__ void __launch_bounds__(cols::kANT, 2) b_cols_spmm_kernel(const BatchG
 // Column-block form: the epilogue over (problem, I, J, pair) items.
 template <int STAGE>
 __global__ void __launch_bounds__(cols::kENT, 3) b_cols_epi_kernel(const BatchGraph *gs, const Ctl *ctls,
-                                                                 const int4 *items, int nitems) {
+                                                                 const int4 *items, const Counts *cn) {
+    const int nitems = cn->b;
+    if ((int)blockIdx.x >= nitems) {
+        tma::grid_dependency_wait();  // a launch without items still ends after the ones before it
+        return;
+    }
     __shared__ __align__(16) float sX1[mixed::TS * mixed::LDX];
     __shared__ __align__(16) float sX2[mixed::TS * mixed::LDX];
     __shared__ __align__(16) float sO[4 * mixed::TS * mixed::LDO];
@@ -305,6 +331,7 @@ int np_class(int np) {
 }
 
 struct Lists {
+    Counts *counts;  // device: the lengths below
     int *act;      // device, active problem indices
     int4 *items;   // device, (problem, I, J, pair index) of the active problems
     int nact, nitems;
@@ -319,6 +346,7 @@ struct Lists {
 
 // Device buffers one set of lists is uploaded into.
 struct ListBufs {
+    Counts *counts = nullptr;
     int *act = nullptr;
     int4 *items = nullptr, *items_a = nullptr, *items_b = nullptr, *items_t = nullptr;
 };
@@ -333,11 +361,11 @@ void launch_refresh(const BatchGraph *gs, const Lists &L, int max_np, cudaStream
                     const uint8_t *due = nullptr) {
     if (L.nact == 0) return;
     const dim3 eg(elem_chunks(max_np), L.nact);
-    b_trace_kernel<<<L.nact, 256, 0, s>>>(gs, L.act, due);
-    b_normalize_kernel<<<eg, 256, 0, s>>>(gs, L.act, due);
+    b_trace_kernel<<<L.nact, 256, 0, s>>>(gs, L.act, L.counts, due);
+    b_normalize_kernel<<<eg, 256, 0, s>>>(gs, L.act, L.counts, due);
     b_sparse64_kernel<<<std::min(L.nitems, 152 * 3), sparse64::NTHREADS, sparse64::SMEM_BYTES, s>>>(gs, L.items,
-                                                                                                     L.nitems, due);
-    b_post_kernel<<<eg, 256, 0, s>>>(gs, L.act, due);
+                                                                                                     L.counts, due);
+    b_post_kernel<<<eg, 256, 0, s>>>(gs, L.act, L.counts, due);
     launches += 4;
 }
 
@@ -363,18 +391,18 @@ void launch_stage_b(const BatchGraph *gs, const Ctl *ctls, const Lists &L, cudaS
     for (int c = 0; c < kClasses; ++c)
         if (L.na[c]) {
             launch_dep(b_cols_spmm_kernel<STAGE>, L.grid_a[c], cols::kANT, (size_t)L.smem_a[c], s, gs, ctls,
-                       (const int4 *)L.items_a[c], L.na[c]);
+                       (const int4 *)L.items_a[c], (const Counts *)L.counts, c);
             launches += 1;
             any = true;
         }
     if (any) {
         launch_dep(b_cols_epi_kernel<STAGE>, std::min(L.nb, 152 * 3), cols::kENT, 0, s, gs, ctls,
-                   (const int4 *)L.items_b, L.nb);
+                   (const int4 *)L.items_b, (const Counts *)L.counts);
         launches += 1;
     }
     if (L.nt) {
         b_stage_mixed_kernel<STAGE><<<std::min(L.nt, 152 * 3), kStageNT, mixed::kMixedDynSmem, s>>>(gs, L.items_t,
-                                                                                                 L.nt);
+                                                                                                 L.counts);
         launches += 1;
     }
 }
@@ -486,6 +514,8 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     std::vector<std::vector<int2>> segs(G);
     std::vector<double> hdt(G);
     std::vector<int64_t> msub(G);
+    std::vector<double> spread(G, 0.0), cmaxs(G, 0.0);
+    std::vector<size_t> on_device;  // problems whose spectral spread the device forms
     for (size_t g = 0; g < G; ++g) {
         const qpr_problem &p = problems[g];
         if (p.n < 2 || p.n > 65536) return err(QPR_E_ARG, "problem " + std::to_string(g) + ": n outside [2, 65536]");
@@ -503,11 +533,9 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         npairs[g] = T[g] * (T[g] + 1) / 2;
         double cmax = 0.0;
         qpr::column_sums_G(H[g], alpha, np[g], &cmax);
-        const double spread = qpr::estimate_spread(p.n, H[g].hptr, H[g].hcol, H[g].hval);
-        const double rate = (1.0 - p.omega) * spread + 2.0 * p.omega * cmax;
-        const double dmax = rate > 0.0 ? 2.5 / rate : INFINITY;
-        msub[g] = (dt > dmax) ? (int64_t)ceil(dt / dmax) : 1;
-        hdt[g] = dt / (double)msub[g];
+        cmaxs[g] = cmax;
+        if (qpr::spread_on_device(H[g], G > 4)) on_device.push_back(g);
+        else spread[g] = qpr::estimate_spread(H[g]);
     }
 
     // ---- arena layout (elements), every sub-array aligned to 64 elements ----
@@ -552,6 +580,7 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     size_t nkh = 0, nci = 0, npc = 0, nxc = 0, na_max = 0;
     int smem_a = 0;
     int smem_class[qpr::kClasses] = {};
+    size_t class_units[qpr::kClasses] = {}, class_off[qpr::kClasses] = {};  // a class's units keep their place
     // Row splits: one where it fits and the batch fills the SMs with many
     // problems; in a small batch, as many as bring a unit's entries down to an
     // even share, with no more units than two CTAs per SM take at once (a
@@ -587,9 +616,12 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         oxc[g] = nxc;
         nxc += qpr::align_up(2 * (size_t)np[g] * np[g], 64);
         na_max += (size_t)(np[g] / qpr::cols::kCW) * pl.splits;
+        class_units[qpr::np_class(np[g])] += (size_t)(np[g] / qpr::cols::kCW) * pl.splits;
         smem_a = std::max(smem_a, pl.smem);
         smem_class[qpr::np_class(np[g])] = std::max(smem_class[qpr::np_class(np[g])], pl.smem);
     }
+
+    for (int c = 1; c < qpr::kClasses; ++c) class_off[c] = class_off[c - 1] + class_units[c - 1];
 
     qpr::BatchMem mem;
     double *dD = nullptr;
@@ -618,6 +650,8 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     BCUDA(mem.alloc(&dG, G));
     qpr::ListBufs gbuf, abuf;  // lists of the captured graph; lists of ad-hoc launches (confirming refreshes)
     uint8_t *dDue = nullptr;
+    BCUDA(mem.alloc(&gbuf.counts, 1));
+    BCUDA(mem.alloc(&abuf.counts, 1));
     BCUDA(mem.alloc(&gbuf.act, G));
     BCUDA(mem.alloc(&gbuf.items, total_pairs));
     BCUDA(mem.alloc(&abuf.act, G));
@@ -772,7 +806,6 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         Ctl &k = hCtl[g];
         k.max_steps = max_steps;
         k.tol = tol;
-        k.dt = hdt[g];
         k.scale = 1.0;
         k.resid_exact_step = -1;
     }
@@ -794,6 +827,34 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     }
     BCUDA(cudaMemcpyAsync(dMaps, hMaps.data(), G * sizeof(qpr::ColMaps), cudaMemcpyHostToDevice, s));
     BCUDA(cudaMemcpyAsync(dG, desc.data(), G * sizeof(BatchGraph), cudaMemcpyHostToDevice, s));
+    if (!on_device.empty()) {
+        std::vector<qpr::SpectrumJob> jobs;
+        int max_n = 0;
+        double *dS = nullptr;
+        qpr::SpectrumJob *dJ = nullptr;
+        BCUDA(mem.alloc(&dS, on_device.size()));
+        BCUDA(mem.alloc(&dJ, on_device.size()));
+        for (size_t k = 0; k < on_device.size(); ++k) {
+            const qpr::DevOps &ops = desc[on_device[k]].ops;
+            jobs.push_back({ops.n, ops.h_ptr, ops.h_col, ops.h_val, dS + k});
+            max_n = std::max(max_n, ops.n);
+        }
+        std::vector<double> raw(jobs.size());
+        BCUDA(cudaMemcpyAsync(dJ, jobs.data(), jobs.size() * sizeof(jobs[0]), cudaMemcpyHostToDevice, s));
+        BCUDA(qpr::spectral_spread(dJ, (int)jobs.size(), max_n, jobs[0], s));
+        BCUDA(cudaMemcpyAsync(raw.data(), dS, raw.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
+        BCUDA(cudaStreamSynchronize(s));
+        for (size_t k = 0; k < on_device.size(); ++k)
+            spread[on_device[k]] = qpr::bounded_spread(H[on_device[k]], raw[k]);
+    }
+    for (size_t g = 0; g < G; ++g) {
+        const double omega = problems[g].omega;
+        const double rate = (1.0 - omega) * spread[g] + 2.0 * omega * cmaxs[g];
+        const double dmax = rate > 0.0 ? 2.5 / rate : INFINITY;
+        msub[g] = (dt > dmax) ? (int64_t)ceil(dt / dmax) : 1;
+        hdt[g] = dt / (double)msub[g];
+        hCtl[g].dt = hdt[g];
+    }
     BCUDA(cudaMemcpyAsync(dCtl, hCtl, G * sizeof(Ctl), cudaMemcpyHostToDevice, s));
     int64_t launches = 0;
     // ---- initial states ----
@@ -838,19 +899,26 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         L.items = bufs.items;
         L.nact = (int)list.size();
         L.nitems = (int)items.size();
-        size_t off = 0;
+        L.counts = bufs.counts;
+        qpr::Counts cn{};
+        static_assert(qpr::kClasses == 2, "Counts");
         for (int c = 0; c < qpr::kClasses; ++c) {
-            L.items_a[c] = bufs.items_a + off;
+            L.items_a[c] = bufs.items_a + class_off[c];
             L.na[c] = (int)items_cls[c].size();
             L.smem_a[c] = smem_class[c];
             L.grid_a[c] = std::max(1, std::min(L.na[c], sms * class_ctas[c]));
-            off += items_cls[c].size();
+            cn.a[c] = L.na[c];
         }
         L.items_b = bufs.items_b;
         L.items_t = bufs.items_t;
         L.nb = (int)items_b.size();
         L.nt = (int)items_t.size();
-        cudaError_t e = cudaMemcpyAsync(bufs.act, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, s);
+        cn.act = L.nact;
+        cn.items = L.nitems;
+        cn.b = L.nb;
+        cn.t = L.nt;
+        cudaError_t e = cudaMemcpyAsync(bufs.counts, &cn, sizeof(cn), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(bufs.act, list.data(), list.size() * sizeof(int), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(bufs.items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, s);
         for (int c = 0; c < qpr::kClasses && e == cudaSuccess; ++c)
@@ -879,8 +947,10 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     // its due flag is set; the host writes the flags before each launch) and
     // `block` steps, over the lists of the active set at capture time.
     // Problems that stop later keep their items in the lists (their kernels
-    // return at once, the device retires them) until the lists are rebuilt
-    // and the graph recaptured, once the active set has shrunk by a quarter.
+    // return at once, the device retires them) until the lists are rebuilt,
+    // once the active set has shrunk by a quarter; the graph, whose grids are
+    // those of the first lists, reads their lengths from device memory
+    // (capturing it anew with smaller grids gained nothing).
     qpr::Lists LG{};
     cudaGraphExec_t gexec = nullptr;
     struct GraphGuard {
@@ -890,17 +960,15 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         }
     } gguard{&gexec};
     int64_t graph_launches = 0;
-    size_t captured = 0;
+    size_t captured = 0;  // active problems when the lists were made
     std::vector<uint8_t> hDue(G, 0);
-    auto recapture = [&]() -> cudaError_t {
-        if (gexec) {
-            cudaGraphExecDestroy(gexec);
-            gexec = nullptr;
-        }
-        cudaError_t e = make_lists(active, gbuf, LG);
-        if (e != cudaSuccess) return e;
+    auto relist = [&]() -> cudaError_t {
         captured = active.size();
-        graph_launches = 0;
+        return make_lists(active, gbuf, LG);
+    };
+    auto capture = [&]() -> cudaError_t {
+        cudaError_t e = relist();
+        if (e != cudaSuccess) return e;
         cudaGraph_t gr = nullptr;
         e = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return e;
@@ -913,7 +981,7 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         if (e != cudaSuccess) gexec = nullptr;
         return e;
     };
-    BCUDA(recapture());
+    BCUDA(capture());
     while (!active.empty()) {
         qpr::NvtxRange nvtx_block("batch block");
         for (int g : active) hDue[g] = due[g] ? 1 : 0;
@@ -967,7 +1035,7 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         }
         std::sort(keep.begin(), keep.end());
         active.swap(keep);
-        if (!active.empty() && 4 * active.size() <= 3 * captured) BCUDA(recapture());
+        if (!active.empty() && 4 * active.size() <= 3 * captured) BCUDA(relist());
     }
 
     // ---- results ----

@@ -511,11 +511,36 @@ qpr_status run_rkf45(qpr_ctx *ctx, double h0, double step_tol, double hmax, doub
 
 namespace qpr {
 
+static double gershgorin(const HostOps &h) {
+    double g = 0.0;
+    for (int64_t i = 0; i < h.n; ++i) {
+        double r = 0.0;
+        for (int64_t q = h.hptr[i]; q < h.hptr[i + 1]; ++q) r += fabs(h.hval[q]);
+        g = std::max(g, r);
+    }
+    return g;
+}
+
+double bounded_spread(const HostOps &h, double raw) { return std::min(raw, 2.0 * gershgorin(h)); }
+
+// From 8000 nonzeros on (800 host sweeps against 800 products of 4 us: a
+// context at N = 300 with 4800 nonzeros 3.2 ms here, 4.5 there; at N = 922 with
+// 14700 10.3 and 6.4), in a batch from 500 (its problems run side by side),
+// and where eight products without rescaling keep the vector in range.
+bool spread_on_device(const HostOps &h, bool many) {
+    if (h.hval.size() < (many ? 500 : 8000) || h.n > kSpectrumMaxN) return false;
+    const double g = gershgorin(h);
+    return g > 1e-15 && g < 1e15;
+}
+
 // Power iteration for the extreme eigenvalues of the symmetric CSR matrix
 // H; returns an estimate of lambda_max - lambda_min (with a 2% margin, and
 // never above the Gershgorin bound).
-double estimate_spread(int64_t n, const std::vector<int64_t> &ptr, const std::vector<int> &col,
-                       const std::vector<double> &val) {
+double estimate_spread(const HostOps &h) {
+    const int64_t n = h.n;
+    const std::vector<int64_t> &ptr = h.hptr;
+    const std::vector<int> &col = h.hcol;
+    const std::vector<double> &val = h.hval;
     if (val.empty()) return 0.0;
     auto matvec = [&](const std::vector<double> &x, std::vector<double> &y, double shift) {
         for (int64_t i = 0; i < n; ++i) {
@@ -542,16 +567,9 @@ double estimate_spread(int64_t n, const std::vector<int64_t> &ptr, const std::ve
         }
         return lam;
     };
-    double gersh = 0.0;
-    for (int64_t i = 0; i < n; ++i) {
-        double r = 0.0;
-        for (int64_t q = ptr[i]; q < ptr[i + 1]; ++q) r += fabs(val[q]);
-        gersh = std::max(gersh, r);
-    }
     const double l1 = dominant(0.0);
     const double l2 = dominant(l1);  // eigenvalue of H - l1 I farthest from 0
-    double spread = fabs(l2) * 1.02 + 1e-12;
-    return std::min(spread, 2.0 * gersh);
+    return bounded_spread(h, fabs(l2) * 1.02 + 1e-12);
 }
 
 void set_create_error(const std::string &msg) { g_create_error = msg; }
@@ -862,7 +880,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
                      (o.backend == QPR_BACKEND_AUTO && (double)hval.size() >= (double)n * (double)n / 8.0));
     if (tc) ctx->np = (int)(((n + qpr::kTileTc - 1) / qpr::kTileTc) * qpr::kTileTc);
     ctx->nnz = (int)hval.size();
-    ctx->spread = qpr::estimate_spread(n, hptr, hcol, hval);
+    if (!qpr::spread_on_device(hops)) ctx->spread = qpr::estimate_spread(hops);
     if (o.backend == QPR_BACKEND_AUTO)
         ctx->backend = ((double)hval.size() < (double)n * (double)n / 8.0) ? QPR_BACKEND_SPARSE : QPR_BACKEND_DENSE;
     else
@@ -1089,6 +1107,13 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     CREATE_CUDA(cudaMalloc(&ctx->d_p, n * sizeof(double)));
     if (n <= qpr::kPrClusterMaxN) CREATE_CUDA(cudaMalloc(&ctx->d_pr, ((size_t)n + qpr::kPrState) * sizeof(double)));
     CREATE_CUDA(cudaMallocHost(&ctx->h_ctl, sizeof(Ctl)));
+    if (qpr::spread_on_device(hops)) {
+        const qpr::SpectrumJob job{(int)n, ctx->d_hptr, ctx->d_hcol, ctx->d_hval, ctx->d_p};
+        CREATE_CUDA(qpr::spectral_spread(nullptr, 0, (int)n, job, nullptr));
+        double raw = 0.0;
+        CREATE_CUDA(cudaMemcpy(&raw, ctx->d_p, sizeof(raw), cudaMemcpyDeviceToHost));
+        ctx->spread = qpr::bounded_spread(hops, raw);
+    }
     CREATE_CUDA(cudaStreamCreateWithFlags(&ctx->stream, cudaStreamNonBlocking));
     CREATE_CUDA(cudaEventCreateWithFlags(&ctx->ev, cudaEventDisableTiming));
 #undef CREATE_CUDA

@@ -447,7 +447,20 @@ cudaError_t init_batch();
 cudaError_t set_bcols_smem(int bytes);
 // Resident CTAs per SM of the batched SpMM with `bytes` of dynamic shared memory.
 cudaError_t bcols_ctas_per_sm(int bytes, int *ctas);
-double estimate_spread(int64_t n, const std::vector<int64_t> &ptr, const std::vector<int> &col,
-                       const std::vector<double> &val);
+// Estimate of lambda_max - lambda_min of H (2% margin, at most twice the
+// Gershgorin radius): power iteration on the host, or, where spread_on_device
+// says so, by spectrum.cu (`raw` its result).
+double estimate_spread(const HostOps &h);
+bool spread_on_device(const HostOps &h, bool many = false);
+double bounded_spread(const HostOps &h, double raw);
+struct SpectrumJob {
+    int n;
+    const int *h_ptr, *h_col;
+    const double *h_val;
+    double *out;
+};
+// `count` jobs in device memory (or `one`, jobs null), n <= max_n each.
+constexpr int kSpectrumMaxN = 8192;
+cudaError_t spectral_spread(const SpectrumJob *jobs, int count, int max_n, const SpectrumJob &one, cudaStream_t s);
 
 }  // namespace qpr
