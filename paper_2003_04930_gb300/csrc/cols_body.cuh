@@ -26,6 +26,8 @@
 // each to the least loaded warp.
 #pragma once
 
+#include <type_traits>
+
 #include "mixed_body.cuh"
 
 namespace qpr {
@@ -222,47 +224,56 @@ __device__ __forceinline__ void narrow_bundles(const float *__restrict__ sD, con
     const int o0 = 4 * c0, o1 = 4 * c1;
     float *__restrict__ X0 = X + (c0 < 4 ? 0 : plane) + J * kCW + 4 * (c0 & 3);
     float *__restrict__ X1 = X + (c1 < 4 ? 0 : plane) + J * kCW + 4 * (c1 & 3);
-    for (int b = b0; b < b1; ++b) {
-        const int4 *bd = sP + kBundleInt4 * (b - p_base);
+    const int4 *bd = sP + kBundleInt4 * (b0 - p_base);
+    for (int b = b0; b < b1; ++b, bd += kBundleInt4) {
         const int4 d0 = bd[0];
+        // this quad's row slot, read ahead of its use
+        const int slot = reinterpret_cast<const int *>(bd + 1)[quad];
         const int2 *__restrict__ kh = sKH + d0.x + quad;
         const int T = d0.y;
         float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0;
         int t = 0;
-        // UNROLL rounds at a time: their entries, then their row reads, then
-        // the FMAs in round order (the same sums as one round at a time)
-        for (; UNROLL > 1 && t + UNROLL <= T; t += UNROLL) {
-            int2 e[UNROLL];
-            float4 v0[UNROLL], v1[UNROLL];
+        // rounds UNROLL at a time, then half as many, ... then one: their
+        // entries, then their row reads, then the FMAs in round order (the
+        // same sums as one round at a time). Most rows have a few rounds, and
+        // one at a time after the last full block each waited for its own
+        // shared-memory latency, as did the row slot read at the end: steady
+        // state at N = 922 114.9 -> 110.1 ms, N = 700 87.3 -> 84.6, N = 1400
+        // 357 -> 345, RKF45 at N = 922 35.3 -> 34.3 (blocks of 8 or 6: N = 500
+        // 1.7% slower).
+        auto rounds = [&](auto count) {
+            constexpr int U = decltype(count)::value;
+            int2 e[U];
+            float4 v0[U], v1[U];
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) e[u] = kh[kNarrowRows * (t + u)];
+            for (int u = 0; u < U; ++u) e[u] = kh[kNarrowRows * (t + u)];
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) {
+            for (int u = 0; u < U; ++u) {
                 const float *__restrict__ row = sD + e[u].x * kRowFloats;
                 v0[u] = *reinterpret_cast<const float4 *>(row + o0);
                 v1[u] = *reinterpret_cast<const float4 *>(row + o1);
             }
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) {
+            for (int u = 0; u < U; ++u) {
                 a0 = f4fma(__int_as_float(e[u].y), v0[u], a0);
                 a1 = f4fma(__int_as_float(e[u].y), v1[u], a1);
             }
-        }
-#pragma unroll 1
-        for (; t < T; ++t) {
-            const int2 e = kh[kNarrowRows * t];
-            const float hv = __int_as_float(e.y);
-            const float *__restrict__ row = sD + e.x * kRowFloats;
-            a0 = f4fma(hv, *reinterpret_cast<const float4 *>(row + o0), a0);
-            a1 = f4fma(hv, *reinterpret_cast<const float4 *>(row + o1), a1);
-        }
+            t += U;
+        };
+        while (t + UNROLL <= T) rounds(std::integral_constant<int, UNROLL>{});
+        if constexpr (UNROLL > 4)
+            if (t + 4 <= T) rounds(std::integral_constant<int, 4>{});
+        if constexpr (UNROLL > 2)
+            if (t + 2 <= T) rounds(std::integral_constant<int, 2>{});
+        if constexpr (UNROLL > 1)
+            if (t < T) rounds(std::integral_constant<int, 1>{});
         if (d0.z & kPieceLong) {
             // chunks 2l and 2l + 1, then the sum over the 8 quads
             float4 u0 = par ? a1 : a0, u1 = par ? a0 : a1;
             u0 = mixed::f4xor(mixed::f4xor(mixed::f4xor(u0, 4), 8), 16);
             u1 = mixed::f4xor(mixed::f4xor(mixed::f4xor(u1, 4), 8), 16);
             if (quad == 0) {
-                const int row = bd[1].x;
+                const int row = slot;
                 if (d0.z & kPiecePart) {
                     *reinterpret_cast<float4 *>(parts + row * kRowFloats + 8 * l) = u0;
                     *reinterpret_cast<float4 *>(parts + row * kRowFloats + 8 * l + 4) = u1;
@@ -273,7 +284,7 @@ __device__ __forceinline__ void narrow_bundles(const float *__restrict__ sD, con
                 }
             }
         } else {
-            const int row = pick(bd[1 + (quad >> 2)], quad & 3);
+            const int row = slot;
             if (row >= 0) {
                 *reinterpret_cast<float4 *>(X0 + (size_t)row * np) = a0;
                 *reinterpret_cast<float4 *>(X1 + (size_t)row * np) = a1;
