@@ -14,7 +14,7 @@ the slowest rank's time divided by the solves of all ranks.
 
 Besides the timed steps, rank 0 adds: the roofline of the dominant kernel
 (each kernel timed alone by qpr_profile_step), the exact FP64 sparse form and
-the plain dense FP64 (DMMA) form on the same problem, the learned warm start,
+the plain dense FP64 form (exact digit products) on the same problem, the learned warm start,
 an end-to-end solve from pinned host memory, the same comparison at N = 4096
 (`n4096`), one 512-graph batched solve (`batch512`) and the CPU oracle.
 
@@ -360,7 +360,7 @@ def run_ours(a):
     # steady-state populations and of the classical PageRank vector, both on the GPU
     line["hubs"] = hub_report(s, rho_solved)
 
-    # the plain dense FP64 (DMMA) form on the same problem: s/step x steps
+    # the plain dense FP64 form (exact digit products) on the same problem: s/step x steps
     if not a.no_dense_projection and s.backend != qpr.QPR_BACKEND_DENSE:
         line["plain_fp64_dense"] = dense_projection(g, a.omega, local, rho, a.dt, steps_conv, peaks, peak_src)
 
@@ -476,7 +476,7 @@ def hub_report(s, rho_ss, c=10.0, top=10):
 
 def form_name(s, prec):
     from paper_2003_04930_gb300 import qpr
-    form = {(qpr.QPR_FP64, 1): "fp64 dense DMMA", (qpr.QPR_FP64, 2): "fp64 sparse CSR",
+    form = {(qpr.QPR_FP64, 1): "fp64 dense digits", (qpr.QPR_FP64, 2): "fp64 sparse CSR",
             (qpr.QPR_MIXED, 1): "mixed: split-BF16 tcgen05 GEMM deltas (FP32 accumulate) + fp64 "
                                 "reference/accumulation/residual",
             (qpr.QPR_MIXED, 2): "mixed: fp32 sparse CSR deltas (tile pairs) + float-float delta "
@@ -536,7 +536,7 @@ def roofline(s, g, n, prof, peaks, peak_src, prec, chain=None):
         flops = 6 * 2.0 * npad * (2 * npad) * npad
         ach = flops / (prof["product_ms"] * 1e-3) / 1e12
         return {"bound": "tensor", "achieved": ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
-                "frac": ach / peaks["bf16_tflops"], "traffic": None, "kernel": "stage_mixed_tc_kernel (tcgen05)",
+                "frac": ach / peaks["bf16_tflops"], "traffic": None, "kernel": "mixed_gemm_kernel (tcgen05)",
                 "alg_flops_per_launch": flops, "launch_ms": prof["product_ms"],
                 "peak_source": f"bf16_tflops of {peak_src}"}
     if s.backend == qpr.QPR_BACKEND_SPARSE and prec == qpr.QPR_MIXED and s.sparse_form != qpr.QPR_SPARSE_FORM_TILES:
@@ -581,13 +581,15 @@ def roofline(s, g, n, prof, peaks, peak_src, prec, chain=None):
     fp64_peak = peaks["bf16_tflops"] * NOMINAL_FP64_OVER_BF16
     ach = flops / (prof["product_ms"] * 1e-3) / 1e12
     return {"bound": "tensor", "achieved": ach, "peak": fp64_peak, "unit": "TFLOP/s",
-            "frac": ach / fp64_peak, "traffic": None, "kernel": "stage_fp64_kernel (DMMA)",
+            "frac": ach / fp64_peak, "traffic": None, "kernel": "digits_gemm_kernel (tcgen05, exact FP16 digit products)",
+            "note": "4 N^3 FP64 flops delivered over the whole stage (digits, product, epilogue); the tensor cores "
+                    "form them from integer digits, so the FP64 pipe's peak is no bound",
             "alg_flops_per_launch": flops, "launch_ms": prof["product_ms"],
             "peak_source": f"bf16_tflops of {peak_src} x nominal FP64/BF16 ratio 1.25/2250"}
 
 
 def dense_projection(g, omega, local, rho, dt, steps_conv, peaks, peak_src, prof_steps=3):
-    """The plain dense FP64 (DMMA) form on the same problem: its step time
+    """The plain dense FP64 form (exact digit products on the tensor cores) on the same problem: its step time
     from qpr_profile_step times the step count of the solve (projected)."""
     from paper_2003_04930_gb300 import Solver, qpr
     sd = Solver.from_edges(g, alpha=0.85, omega=omega, backend=qpr.QPR_BACKEND_DENSE, device=local)
@@ -766,7 +768,7 @@ def large_case(a, local, peaks, peak_src, flush):
     """The metric's second size: the same generator at N = 4096 (seed 3),
     omega = 0.8. Mixed cold and warm-started solves (one timed each after one
     untimed), one FP64 sparse solve (the exact form, also the reference of
-    the error), the plain dense FP64 DMMA form projected from one profiled
+    the error), the plain dense FP64 form projected from one profiled
     step, and the roofline of the gather SpMM and the epilogue."""
     import torch
     from paper_2003_04930_gb300 import Solver, graphs, qpr

@@ -568,7 +568,7 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     e = cudaMemcpy(dw->erow, p.erow.data(), p.erow.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
     split_h_kernel<<<std::min(ops.n, 4096), 128>>>(ops, p.b, p.sh, dw->erow, hd);
-    e = cudaDeviceSynchronize();
+    e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return e;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc) return cudaErrorNotSupported;
