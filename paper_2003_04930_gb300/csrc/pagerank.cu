@@ -15,6 +15,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <utility>
 #include <vector>
 
@@ -297,6 +298,40 @@ cudaError_t pagerank(const DevOps &ops, double tol, int64_t max_iter, double *sc
     if (iters) *iters = it;
     if (delta_out) *delta_out = d;
     return e;
+}
+
+// Which form: the cluster has 32 schedulers, the grid up to 1216 but a launch
+// per iteration and the sums over all nodes in every CTA. Per iteration the
+// cluster takes about 3 us and 10.5 ns for each FP64 warp instruction of its
+// busiest CTA (counted below from the rows' lengths), the grid 13 us and 4.5 ns
+// per node. Measured, cluster against grid, us per iteration: sparse
+// (heavy-tailed, 8 links a node) N = 922 3.2 and 14.6, N = 8192 15.6 and 48;
+// links with p = 0.25 N = 700 12.1 and 15.6, N = 900 18.5 and 16.0, N = 2000 68
+// and 27, N = 4000 181 and 43; p = 0.005 N = 8192 35 and 49; 60 rows of all
+// nodes N = 2000 39 and 28. The cluster form also takes the columns of S to
+// sum to one, which they do unless an out-degree overflows.
+bool pagerank_in_cluster(const HostOps &h) {
+    const int n = (int)h.n;
+    if (n > kPrClusterMaxN) return false;
+    for (double d : h.outdeg)
+        if (!std::isfinite(d)) return false;
+    const int per = (n + kPrCtas - 1) / kPrCtas;
+    int64_t most = 0;
+    for (int r0 = 0; r0 < n; r0 += per) {
+        const int r1 = std::min(n, r0 + per);
+        int64_t work = 6 * ((r1 - r0 + 31) / 32);
+        for (int b = r0; b < r1; b += 8) {
+            int quad = 0;  // rounds of the longest short row of a warp's eight
+            for (int i = b; i < std::min(r1, b + 8); ++i) {
+                const int len = h.sptr[i + 1] - h.sptr[i];
+                if (len > kPrLong) work += (len + 31) / 32 + 5;
+                else quad = std::max(quad, (len + 3) / 4);
+            }
+            work += quad + 2;
+        }
+        most = std::max(most, work);
+    }
+    return (double)most <= 950.0 + 0.43 * n;
 }
 
 cudaError_t pagerank_cluster(const DevOps &ops, double tol, int64_t max_iter, double *scratch, double *pi_out_dev,

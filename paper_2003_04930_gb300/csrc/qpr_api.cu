@@ -65,7 +65,7 @@ struct qpr_ctx {
     int4 *d_epi_pairs = nullptr, *d_pairs64 = nullptr;
     Ctl *d_ctl = nullptr;
     double *d_io = nullptr;     // staging for host density matrices (interleaved)
-    double *d_pr = nullptr;     // PageRank: the iterate and its state (kPrScratch)
+    double *d_pr = nullptr;     // PageRank in one cluster: the iterate and its state (null: the grid form)
     double *d_p = nullptr;      // populations staging
     float *d_rkf = nullptr;     // RKF45: D1, Dlo1, acc, Flo (2 planes each), the two compact diagonals
     cudaGraphExec_t graph_rkf = nullptr;  // RKF45: refresh + ref_refresh attempts
@@ -1105,7 +1105,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
     CREATE_CUDA(cudaMemset(ctx->d_ctl, 0, sizeof(Ctl)));
     CREATE_CUDA(cudaMalloc(&ctx->d_io, (size_t)n * n * 2 * sizeof(double)));
     CREATE_CUDA(cudaMalloc(&ctx->d_p, n * sizeof(double)));
-    if (n <= qpr::kPrClusterMaxN) CREATE_CUDA(cudaMalloc(&ctx->d_pr, ((size_t)n + qpr::kPrState) * sizeof(double)));
+    if (qpr::pagerank_in_cluster(hops)) CREATE_CUDA(cudaMalloc(&ctx->d_pr, ((size_t)n + qpr::kPrState) * sizeof(double)));
     CREATE_CUDA(cudaMallocHost(&ctx->h_ctl, sizeof(Ctl)));
     if (qpr::spread_on_device(hops)) {
         const qpr::SpectrumJob job{(int)n, ctx->d_hptr, ctx->d_hcol, ctx->d_hval, ctx->d_p};
@@ -1662,7 +1662,7 @@ qpr_status qpr_pagerank(qpr_ctx *ctx, double tol, int64_t max_iter, double *pi, 
     const int64_t n = ctx->n;
     int64_t it = 0, launches = 0;
     double delta = 0.0;
-    if (n <= qpr::kPrClusterMaxN) {
+    if (ctx->d_pr) {
         QPR_CUDA(ctx, qpr::pagerank_cluster(ctx->ops, tol, max_iter, ctx->d_pr, ctx->d_p, &it, &delta, &launches, ctx->stream));
     } else {
         QPR_CUDA(ctx, qpr::pagerank(ctx->ops, tol, max_iter, ctx->d_io, ctx->d_p, &it, &delta, ctx->stream));

@@ -390,8 +390,10 @@ cudaError_t pagerank(const DevOps &ops, double tol, int64_t max_iter, double *sc
                      int64_t *iters, double *delta_out, cudaStream_t s);
 // The same for n <= kPrClusterMaxN in one cluster per graph, up to a few
 // thousand iterations per launch. scratch: n + kPrState doubles.
+// pagerank_in_cluster: whether this form is the faster one for a graph.
 constexpr int kPrClusterMaxN = 8192;
 constexpr int kPrState = 4;
+bool pagerank_in_cluster(const HostOps &h);
 cudaError_t pagerank_cluster(const DevOps &ops, double tol, int64_t max_iter, double *scratch, double *pi_out_dev,
                              int64_t *iters, double *delta_out, int64_t *launches, cudaStream_t s);
 // A fixed number of power iterations for `count` graphs of at most max_n <=
