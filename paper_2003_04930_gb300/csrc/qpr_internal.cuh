@@ -257,14 +257,16 @@ struct DigitWork {
     void *yd;             // FP16 digits of the stage input [s][2 planes][np][np]
     int *ecol;            // [2 planes][np]: the exponent of the first digit's unit of a row of Y
     int *erow;            // np
-    double *x;            // [H Re Y ; -H Im Y], 2 planes
+    double *x;            // [H Re Y ; -H Im Y] without the diagonal of Y, 2 planes
+    const double *h;      // H, np x np
+    double *diag;         // the diagonal of the stage input, np
 };
 struct DigitMaps {
     CUtensorMap h, y;
 };
 // False if no digit width keeps the sums exact (stage_fp64.cu serves then).
 bool plan_digits(const HostOps &h, DigitPlan &p);
-// FP16 values of the digit planes; ints: 3 np, x: 2 np^2.
+// FP16 values of the digit planes; ints: 3 np, x: 3 np^2 + np.
 size_t digits_half_count(const DigitPlan &p, int np);
 cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *halves, int *ints, double *x, DigitWork *dw,
                         DigitMaps *maps);

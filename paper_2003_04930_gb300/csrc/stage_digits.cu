@@ -7,17 +7,28 @@
 // about 1900. The FP64 tensor instruction (stage_fp64.cu) took 616 us per
 // stage at N = 500 (4.2 ms at N = 922), one 32 x 32 tile pair per CTA; this
 // form takes 27 us at N = 500 with unit weights and 363 us at N = 922 with
-// lognormal ones. Here
-// every entry is written as
+// lognormal ones. Here every entry off the diagonal is written as
 //     Y_jk = 2^(ec_j) sum_s y_s(j, k) 2^(-b s),   s < S,  |y_s| <= 2^(b-1),
-// with integers y_s (exact in FP16) and ec_j from the largest entry of row j,
-// so S b >= 64 bits of every column of Y enter the product, and H likewise
-// (one digit when its entries are small multiples of one power of two, as
-// with unit weights; else S digits of its own row). The products of digits i
-// and j with i + j = d share a weight, and all of them are summed in one FP32
-// accumulator that stays an integer below 2^24: exact in any order. What is
-// dropped is below 2^-64 of the column's largest entry, so X is the FP64
-// product with one rounding: closer to the exact one than FMA chains are.
+// with integers y_s (exact in FP16) and ec_j from the largest entry of row j
+// off the diagonal, so S b >= 64 bits of every column of Y enter the product,
+// and H likewise (one digit when its entries are small multiples of one power
+// of two, as with unit weights; else S digits of its own row). The products of
+// digits i and j with i + j = d share a weight, and all of them are summed in
+// one FP32 accumulator that stays an integer below 2^24: exact in any order.
+//
+// What is left out: the digits after the S-th and, where H has several, the
+// pairs with i + j >= S, together at most
+//     5 S 2^(-S b) nnz(row i of H) max|H_i| max|Y_j|
+// of X_ij, max|Y_j| the largest entry of column j off the diagonal; then one
+// rounding (and at b = 10 one of the low half's 54 bits). The bound is relative
+// to these largest entries: an entry of Y further below its column's largest
+// than S b - 53 bits (11 to 19) enters with fewer than FP64's 53 bits. The
+// diagonal, which is what towers over a column in a state with small
+// coherences, therefore stays out of the product and is added exactly by the
+// epilogue as H_ab (Y_bb - Y_aa) (DiagonalTerm): with it in the product,
+// entries of pairs that are not linked were off by up to 1e-13 of their terms
+// with coherences of 1e-5 / N and 1e-10 with 1e-8 / N, now 1e-16 (CPU model, N =
+// 60, lognormal weights; FMA chains 1e-16).
 //
 // Kernels of a stage: split_kernel (digits of the stage input, a row per
 // CTA), digits_gemm_kernel (one 128 x 32 tile of [H Re Y | -H Im Y] per CTA;
@@ -124,10 +135,18 @@ __global__ void __launch_bounds__(128) split_kernel(DevOps ops, Ctl *ctl, const 
     const double2 *src = reinterpret_cast<const double2 *>(y + pl * plane + (size_t)row * np);
     const int k0 = (warp & 1) * 32 + lane, nk = np / 2;
     double2 v[U];
+    // the diagonal entry stays outside the product (DiagonalTerm); the gain and
+    // the epilogue read it from a vector
+    const double yd = threadIdx.x == 0 ? y[(size_t)row * (np + 1)] : 0.0;
+    auto load = [&](int k) {
+        double2 r = k < nk ? src[k] : make_double2(0.0, 0.0);
+        if (k == row >> 1) (row & 1 ? r.y : r.x) = 0.0;
+        return r;
+    };
     unsigned top = 0;
     for (int k = k0; k < nk; k += 64 * U) {
 #pragma unroll
-        for (int i = 0; i < U; ++i) v[i] = (k + 64 * i < nk) ? src[k + 64 * i] : make_double2(0.0, 0.0);
+        for (int i = 0; i < U; ++i) v[i] = load(k + 64 * i);
 #pragma unroll
         for (int i = 0; i < U; ++i)
             top = max(top, max((unsigned)__double2hiint(v[i].x) & 0x7fffffffu, (unsigned)__double2hiint(v[i].y) & 0x7fffffffu));
@@ -138,13 +157,14 @@ __global__ void __launch_bounds__(128) split_kernel(DevOps ops, Ctl *ctl, const 
     top = max(s_top[2 * pl], s_top[2 * pl + 1]);
     const int ea = exp_above(top);
     const int e0 = ea - (B - 1);  // unit of the first digit
+    if (threadIdx.x == 0) dw.diag[row] = yd;
     if ((warp & 1) == 0 && lane == 0) dw.ecol[pl * np + row] = (top >= 0x7ff00000u) ? kNanExp : e0;
     __half2 *dst = reinterpret_cast<__half2 *>(dw.yd) + (pl * plane + (size_t)row * np) / 2;
     const int eu = e0 - B * (S - 1);
     for (int k = k0; k < nk; k += 64 * U) {
         if (nk > 64 * U) {
 #pragma unroll
-            for (int i = 0; i < U; ++i) v[i] = (k + 64 * i < nk) ? src[k + 64 * i] : make_double2(0.0, 0.0);
+            for (int i = 0; i < U; ++i) v[i] = load(k + 64 * i);
         }
 #pragma unroll
         for (int i = 0; i < U; ++i) {
@@ -159,13 +179,15 @@ __global__ void __launch_bounds__(128) split_kernel(DevOps ops, Ctl *ctl, const 
     }
 }
 
-// Digits of the entries of H into the zeroed planes hd [sh][np][np].
-__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd) {
+// Digits of the entries of H into the zeroed planes hd [sh][np][np], and the
+// entries themselves into the zeroed plane hf.
+__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd, double *hf) {
     const size_t plane = (size_t)ops.np * ops.np;
     for (int i = blockIdx.x; i < ops.n; i += gridDim.x)
         for (int q = ops.h_ptr[i] + threadIdx.x; q < ops.h_ptr[i + 1]; q += blockDim.x) {
             int16_t d[kMaxDigits];
             digits_of(ops.h_val[q], erow[i] - b * (sh - 1), sh, b, d);
+            hf[(size_t)i * ops.np + ops.h_col[q]] = ops.h_val[q];
             for (int s = 0; s < sh; ++s) hd[s * plane + (size_t)i * ops.np + ops.h_col[q]] = __short2half_rn(d[s]);
         }
 }
@@ -221,7 +243,7 @@ __device__ __forceinline__ double scaled(double v, int e) {
 template <int S, int B>
 __global__ void __launch_bounds__(GT) digits_gemm_kernel(const __grid_constant__ CUtensorMap tmH,
                                                          const __grid_constant__ CUtensorMap tmY, DevOps ops, Work w,
-                                                         DigitWork dw, int stage, const double *__restrict__ yin) {
+                                                         DigitWork dw, int stage) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint64_t fullA[kMaxRing], emptyA[kMaxRing], fullB[kMaxRing], emptyB[kMaxRing], accum_bar;
     __shared__ uint32_t tmem_base_sh;
@@ -240,7 +262,7 @@ __global__ void __launch_bounds__(GT) digits_gemm_kernel(const __grid_constant__
     if (u >= tiles_m * (2 * np / TN)) {  // a CTA without a tile: a small problem's gain has more rows than its tiles' warps
         tma::grid_dependency_wait();
         tma::launch_dependents();
-        if (warp >= 2) gain64::gain_fp64_body(stage, ops, w, yin, (size_t)np + 1, u, dw.gain_ctas, gain64::Warps<2, GT - 64>{});
+        if (warp >= 2) gain64::gain_fp64_body(stage, ops, w, dw.diag, 1, u, dw.gain_ctas, gain64::Warps<2, GT - 64>{});
         return;
     }
 
@@ -330,7 +352,7 @@ __global__ void __launch_bounds__(GT) digits_gemm_kernel(const __grid_constant__
         if (!ok) atomicExch(&s_fail, 1);
         umma_commit(&accum_bar);
     } else if (warp >= 2 && u < dw.gain_ctas) {
-        gain64::gain_fp64_body(stage, ops, w, yin, (size_t)np + 1, u, dw.gain_ctas, gain64::Warps<2, GT - 64>{});
+        gain64::gain_fp64_body(stage, ops, w, dw.diag, 1, u, dw.gain_ctas, gain64::Warps<2, GT - 64>{});
     }
     __syncwarp();
     const bool ok_acc = !work || mbar_wait(&accum_bar, 0);
@@ -400,12 +422,38 @@ __global__ void __launch_bounds__(GT) digits_gemm_kernel(const __grid_constant__
 
 constexpr int LDX = 2 * kEpiTS + 1;
 constexpr int EPI_BYTES = 2 * kEpiTS * LDX * (int)sizeof(double);
-constexpr int ET = 256;
+// 512 threads, two elements each: a stage takes 22.2, 26.5 and 41.1 us at N =
+// 200, 500 and 700 (unit weights); with 256 it took 22.8, 26.4 and 47.6.
+constexpr int ET = 512;
+
+// The diagonal's part of A_ab - A_ba, which the product leaves out: H_ab (Y_bb -
+// Y_aa). H_ab in registers, the diagonal's entries of rows I and columns J in
+// shared memory (in registers too a stage took 0.3 us longer at N = 500).
+struct DiagonalTerm {
+    static constexpr int E = EpiIn<1, ET>::E;
+    double h[E];
+    const double *sd;  // Y_aa of the 32 rows, then Y_bb of the 32 columns
+
+    __device__ __forceinline__ void load(const DevOps &ops, const DigitWork &d, int I, int J, double *shared) {
+#pragma unroll
+        for (int i = 0; i < E; ++i) {
+            const int ga = I * kEpiTS + (threadIdx.x >> 5) + i * (ET / 32);
+            h[i] = __ldcg(d.h + (size_t)ga * ops.np + J * kEpiTS + (threadIdx.x & 31));
+        }
+        if (threadIdx.x < 2 * kEpiTS)
+            shared[threadIdx.x] = __ldcg(d.diag + (threadIdx.x < kEpiTS ? I : J) * kEpiTS + (threadIdx.x & 31));
+        sd = shared;
+    }
+    __device__ __forceinline__ double operator()(int i, double d) const {
+        const double dy = __dsub_rn(sd[kEpiTS + (threadIdx.x & 31)], sd[(threadIdx.x >> 5) + i * (ET / 32)]);
+        return __fma_rn(h[i], dy, d);
+    }
+};
 
 template <int STAGE>
-__global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, const double *__restrict__ x) {
+__global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, DigitWork d) {
     extern __shared__ __align__(16) double sm[];
-    __shared__ double red[ET / 32], sg[kEpiTS];
+    __shared__ double red[ET / 32], sg[kEpiTS], s_diag[2 * kEpiTS];
     __shared__ int s_done;
     const int I = w.pairs[blockIdx.x].x, J = w.pairs[blockIdx.x].y;
     const bool diag = I == J;
@@ -414,16 +462,18 @@ __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, cons
     double *sX1 = sm, *sX2 = sm + kEpiTS * LDX;
     EpiIn<STAGE, ET> in;
     in.load(ops, w, I, J);
+    DiagonalTerm dg;
+    dg.load(ops, d, I, J, s_diag);
     tma::grid_dependency_wait();
     tma::launch_dependents();
     if (threadIdx.x == 0) s_done = *(volatile int *)&w.ctl->done;
 #pragma unroll
     for (int a = warp; a < kEpiTS; a += ET / 32) {
-        const double *s1 = x + (size_t)(I * kEpiTS + a) * np + J * kEpiTS + lane;
+        const double *s1 = d.x + (size_t)(I * kEpiTS + a) * np + J * kEpiTS + lane;
         sX1[a * LDX + lane] = __ldcg(s1);
         sX1[a * LDX + kEpiTS + lane] = __ldcg(s1 + plane);
         if (!diag) {
-            const double *s2 = x + (size_t)(J * kEpiTS + a) * np + I * kEpiTS + lane;
+            const double *s2 = d.x + (size_t)(J * kEpiTS + a) * np + I * kEpiTS + lane;
             sX2[a * LDX + lane] = __ldcg(s2);
             sX2[a * LDX + kEpiTS + lane] = __ldcg(s2 + plane);
         }
@@ -431,7 +481,7 @@ __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, cons
     if (diag && threadIdx.x < kEpiTS) sg[threadIdx.x] = __ldcg(w.g + I * kEpiTS + threadIdx.x);
     __syncthreads();
     if (s_done) return;
-    stage_epilogue<STAGE, ET>(ops, w, I, J, diag, in, sX1, sX2, LDX, sg, red, blockIdx.x, blockIdx.x == 0);
+    stage_epilogue<STAGE, ET>(ops, w, I, J, diag, in, sX1, sX2, LDX, sg, red, blockIdx.x, blockIdx.x == 0, dg);
 }
 
 template <typename K, typename... A>
@@ -459,7 +509,7 @@ void launch_sb(const DevOps &ops, const Work &w, const DigitWork &d, const Digit
     const double *yin = (STAGE <= 1) ? w.y : (STAGE == 3 ? w.yb : w.ya);
     launch_dep(split_kernel<S, B>, ops.np, 128, 0, s, ops, w.ctl, yin, d);
     const int tiles = ((ops.np + TM - 1) / TM) * (2 * ops.np / TN);
-    launch_dep(digits_gemm_kernel<S, B>, std::max(tiles, d.gain_ctas), GT, (size_t)gemm_smem(d), s, m.h, m.y, ops, w, d, STAGE, yin);
+    launch_dep(digits_gemm_kernel<S, B>, std::max(tiles, d.gain_ctas), GT, (size_t)gemm_smem(d), s, m.h, m.y, ops, w, d, STAGE);
 }
 
 template <int STAGE>
@@ -473,7 +523,7 @@ void launch_t(const DevOps &ops, const Work &w, const DigitWork &d, const DigitM
         case 6: launch_sb<STAGE, 11, 6>(ops, w, d, m, s); break;
         default: launch_sb<STAGE, 13, 5>(ops, w, d, m, s); break;
     }
-    launch_dep(digits_epi_kernel<STAGE>, w.npairs, ET, (size_t)d.epi_smem, s, ops, w, (const double *)d.x);
+    launch_dep(digits_epi_kernel<STAGE>, w.npairs, ET, (size_t)d.epi_smem, s, ops, w, d);
 }
 
 // The candidates: bits per digit and digits (S b >= 64).
@@ -484,13 +534,14 @@ constexpr Cand kCands[] = {{12, 6}, {11, 6}, {10, 7}, {8, 8}, {7, 10}, {6, 11}, 
 
 }  // namespace
 
-// Digits of H. One digit when every entry is k 2^t with |k| <= 2048 (exact in
+// Digits of H. One digit when every entry is k 2^t with |k| < 2048 (exact in
 // FP16); else as many as of Y, of each row by its largest entry. The bits per
 // digit are the most for which no sum of a weight's products can leave the
 // integers an FP32 accumulator holds exactly: 2^(b-1) times the largest row
 // sum of |digits of H| at most 2^24. With unit weights b = 12 up to row sums
-// of 8192; with general weights b = 8 at N = 64, 6 at N = 1000, 5 up to about
-// N = 5000. Beyond that the FP64 tensor kernel stays in use.
+// of 8192; with general weights, whose digits are half their largest on
+// average, b = 8 for rows of up to about 250 nonzeros, 7 up to 800, 6 up to
+// 2900 and 5 up to 10000. Beyond that the FP64 tensor kernel stays in use.
 bool plan_digits(const HostOps &h, DigitPlan &p) {
     const int n = (int)h.n;
     if (h.hval.empty()) return false;
@@ -547,6 +598,8 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     dw->ecol = ints;
     dw->erow = ints + 2 * np;
     dw->x = x;
+    dw->h = x + 2 * plane;
+    dw->diag = x + 3 * plane;
     dw->b = p.b;
     dw->s = p.s;
     dw->sh = p.sh;
@@ -567,7 +620,9 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     if (e != cudaSuccess) return e;
     e = cudaMemcpy(dw->erow, p.erow.data(), p.erow.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
-    split_h_kernel<<<std::min(ops.n, 4096), 128>>>(ops, p.b, p.sh, dw->erow, hd);
+    e = cudaMemset(x + 2 * plane, 0, plane * sizeof(double));
+    if (e != cudaSuccess) return e;
+    split_h_kernel<<<std::min(ops.n, 4096), 128>>>(ops, p.b, p.sh, dw->erow, hd, x + 2 * plane);
     e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return e;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();

@@ -71,16 +71,23 @@ struct EpiIn {
     }
 };
 
+// What the product left out of A_ab - A_ba of an element: nothing here, the
+// diagonal of the stage input in the digit products.
+struct WholeProduct {
+    __device__ __forceinline__ double operator()(int, double d) const { return d; }
+};
+
 // Must be called by all NT threads of the CTA after the X tiles are complete
 // and visible (__syncthreads()). Off the diagonal sX1 is overwritten with the
 // outputs, each by the one thread that reads that place.
 // g: the gain of rows I, read on diagonal pairs. pidx: slot of this tile
 // pair's residual partial; first: the tile pair that advances the step counter
-// at stage 4.
-template <int STAGE, int NT>
+// at stage 4. rest(i, A_ab - A_ba) adds what the product left out.
+template <int STAGE, int NT, typename P = WholeProduct>
 __device__ __forceinline__ void stage_epilogue(const DevOps &ops, const Work &w, int I, int J, bool diag,
                                                const EpiIn<STAGE, NT> &in, double *sX1, const double *sX2, int ldx,
-                                               const double *g, double *red, int pidx, bool first) {
+                                               const double *g, double *red, int pidx, bool first,
+                                               const P &rest = P{}) {
     constexpr int TS = kEpiTS, E = EpiIn<STAGE, NT>::E;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int np = ops.np;
@@ -105,7 +112,7 @@ __device__ __forceinline__ void stage_epilogue(const DevOps &ops, const Work &w,
         const double Aba = X2[b * ldx + a], nBba = X2[b * ldx + TS + a];
         const double omhc = __dmul_rn(hom, __dadd_rn(in.ca[i], in.cb));  // the same for (b, a)
         double kr = __fma_rn(-omhc, in.ir[i], __dmul_rn(-cm, __dadd_rn(nBab, nBba)));
-        const double ki = __fma_rn(-omhc, in.ii[i], __dmul_rn(-cm, __dsub_rn(Aab, Aba)));
+        const double ki = __fma_rn(-omhc, in.ii[i], __dmul_rn(-cm, rest(i, __dsub_rn(Aab, Aba))));
         if (ga == gb) kr = __fma_rn(om, g[a], kr);
         if (STAGE <= 1) nrm = __fma_rn(kr, kr, __fma_rn(ki, ki, nrm));
         double o0 = kr, o1 = ki;
