@@ -515,7 +515,7 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
     std::vector<double> hdt(G);
     std::vector<int64_t> msub(G);
     std::vector<double> spread(G, 0.0), cmaxs(G, 0.0);
-    std::vector<size_t> on_device;  // problems whose spectral spread the device forms
+    std::vector<size_t> on_device, on_host;  // where the problems' spectral spreads are formed
     for (size_t g = 0; g < G; ++g) {
         const qpr_problem &p = problems[g];
         if (p.n < 2 || p.n > 65536) return err(QPR_E_ARG, "problem " + std::to_string(g) + ": n outside [2, 65536]");
@@ -534,9 +534,9 @@ extern "C" qpr_status qpr_batch_steady_state(int64_t count, const qpr_problem *p
         double cmax = 0.0;
         qpr::column_sums_G(H[g], alpha, np[g], &cmax);
         cmaxs[g] = cmax;
-        if (qpr::spread_on_device(H[g], G > 4)) on_device.push_back(g);
-        else spread[g] = qpr::estimate_spread(H[g]);
+        (qpr::spread_on_device(H[g]) ? on_device : on_host).push_back(g);
     }
+    if (!qpr::estimate_spreads(H, on_host, spread)) return err(QPR_E_OOM, "host allocation failed");
 
     // ---- arena layout (elements), every sub-array aligned to 64 elements ----
     std::vector<size_t> od(G), of(G), oi(G), ob(G);

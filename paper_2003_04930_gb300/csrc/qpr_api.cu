@@ -7,10 +7,12 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <chrono>
 #include <cstdlib>
 #include <numeric>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "qpr_internal.cuh"
@@ -525,10 +527,11 @@ double bounded_spread(const HostOps &h, double raw) { return std::min(raw, 2.0 *
 
 // From 8000 nonzeros on (800 host sweeps against 800 products of 4 us: a
 // context at N = 300 with 4800 nonzeros 3.2 ms here, 4.5 there; at N = 922 with
-// 14700 10.3 and 6.4), in a batch from 500 (its problems run side by side),
-// and where eight products without rescaling keep the vector in range.
-bool spread_on_device(const HostOps &h, bool many) {
-    if (h.hval.size() < (many ? 500 : 8000) || h.n > kSpectrumMaxN) return false;
+// 14700 10.3 and 6.4), and where eight products without rescaling keep the
+// vector in range. The two sum in different orders, so the rule is the same
+// for a problem alone and in a batch: both have to take the same substeps.
+bool spread_on_device(const HostOps &h) {
+    if (h.hval.size() < 8000 || h.n > kSpectrumMaxN) return false;
     const double g = gershgorin(h);
     return g > 1e-15 && g < 1e15;
 }
@@ -570,6 +573,32 @@ double estimate_spread(const HostOps &h) {
     const double l1 = dominant(0.0);
     const double l2 = dominant(l1);  // eigenvalue of H - l1 I farthest from 0
     return bounded_spread(h, fabs(l2) * 1.02 + 1e-12);
+}
+
+// A thread for every 4000 nonzeros (about 2 ms of power iteration), 16 at most.
+bool estimate_spreads(const std::vector<HostOps> &h, const std::vector<size_t> &which, std::vector<double> &out) {
+    size_t nnz = 0;
+    for (size_t g : which) nnz += h[g].hval.size();
+    const size_t cpus = std::max(1u, std::thread::hardware_concurrency());
+    const size_t want = std::min({which.size(), nnz / 4000 + 1, cpus, (size_t)16});
+    std::atomic<size_t> next{0};
+    std::atomic<bool> ok{true};
+    auto run = [&] {
+        try {
+            for (size_t k; (k = next++) < which.size();) out[which[k]] = estimate_spread(h[which[k]]);
+        } catch (...) {
+            ok = false;
+        }
+    };
+    std::vector<std::thread> threads;
+    try {
+        threads.reserve(want);
+        while (threads.size() + 1 < want) threads.emplace_back(run);
+    } catch (...) {  // no more threads: the ones there are do the work
+    }
+    run();
+    for (std::thread &t : threads) t.join();
+    return ok;
 }
 
 void set_create_error(const std::string &msg) { g_create_error = msg; }

@@ -455,7 +455,9 @@ cudaError_t bcols_ctas_per_sm(int bytes, int *ctas);
 // Gershgorin radius): power iteration on the host, or, where spread_on_device
 // says so, by spectrum.cu (`raw` its result).
 double estimate_spread(const HostOps &h);
-bool spread_on_device(const HostOps &h, bool many = false);
+bool spread_on_device(const HostOps &h);
+// estimate_spread of the problems `which`, on several host threads (false: out of memory).
+bool estimate_spreads(const std::vector<HostOps> &h, const std::vector<size_t> &which, std::vector<double> &out);
 double bounded_spread(const HostOps &h, double raw);
 struct SpectrumJob {
     int n;
