@@ -238,13 +238,19 @@ QPR_API qpr_status qpr_steady_state(qpr_ctx *ctx, void *rho, double dt, double t
  * Means over all launches of the kind, in milliseconds. */
 typedef struct {
     double product_ms;   /* the H rho product: the column-block SpMM (COLUMNS, COLUMNS_PERSISTENT) or
-                            gather SpMM (COLUMNS_GATHER), whose leading CTAs also form the gain; the fused
-                            stage kernel of the other forms (product and epilogue in one launch) */
-    double epilogue_ms;  /* the epilogue kernel of the two-kernel column-block forms; 0 otherwise */
-    double gain_ms;      /* the gain kernel G p (0 where the product or stage kernel forms the gain) */
+                            gather SpMM (COLUMNS_GATHER), whose leading CTAs also form the gain, and the
+                            product kernel of the mixed dense form likewise; the fused stage kernel of the
+                            other forms (product and epilogue in one launch); QPR_FP64 dense by digits:
+                            the three launches of a stage together; QPR_FP64 with N <= 44: a whole step of
+                            the one launch that runs up to 1024 of them */
+    double epilogue_ms;  /* the epilogue kernel of the two-kernel forms; 0 otherwise */
+    double gain_ms;      /* the gain kernel G p (0 where the product or stage kernel forms the gain, but for
+                            QPR_FP64 sparse: there its stage forms the gain too, and this is the gain kernel
+                            run beside it, which a solve does not launch) */
     double refresh_ms;   /* QPR_MIXED: one exact FP64 reference refresh, all its kernels; 0 otherwise */
     double step_ms;      /* the kernels of one RK4 step run one at a time (the sum of the above) */
-    int32_t launches_per_step;
+    int32_t launches_per_step;  /* of the timed kernels: 8 for QPR_FP64 sparse with the gain kernel (a solve: 4),
+                                   12 for digits, 0 with N <= 44 (less than one) */
     int32_t reserved[3];
 } qpr_profile;
 

@@ -1546,11 +1546,20 @@ qpr_status qpr_profile_step(qpr_ctx *ctx, const void *rho, double dt, int64_t st
     const qpr::Work &w = ctx->work;
     const double *yin[5] = {w.y, w.y, w.ya, w.yb, w.ya};
     int per_step = 0;
+    cudaError_t launched = cudaSuccess;
     if (mixed) {
         st = timed(3, [&] { qpr::launch_mixed_refresh(ctx->ops, ctx->mw, ctx->stream); });
         if (st != QPR_OK) { destroy(); return st; }
     }
-    for (int64_t k = 0; k < steps && st == QPR_OK; ++k) {
+    const bool small = !mixed && ctx->n <= qpr::kSmallMaxN;  // one launch runs many steps
+    for (int64_t left = small ? steps : 0; left > 0 && st == QPR_OK; left -= qpr::kSmallSteps) {
+        const int run = (int)std::min<int64_t>(left, qpr::kSmallSteps);
+        st = timed(0, [&] {
+            launched = qpr::launch_small_rk4(ctx->ops, ctx->work, ctx->nnz, run, ctx->stream);
+        });
+        if (st == QPR_OK && launched != cudaSuccess) st = cuda_fail(ctx, launched, "launch_small_rk4");
+    }
+    for (int64_t k = small ? steps : 0; k < steps && st == QPR_OK; ++k) {
         for (int s = 1; s <= 4 && st == QPR_OK; ++s) {
             if (cols) {
                 st = timed(0, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 1, true); });
@@ -1560,8 +1569,13 @@ qpr_status qpr_profile_step(qpr_ctx *ctx, const void *rho, double dt, int64_t st
             } else if (mixed) {
                 st = timed(0, [&] { qpr::launch_mixed_stage(s, ctx->ops, ctx->mw, ctx->stream, 2, true); });
                 if (k == 0) per_step += 1;
+            } else if (ctx->d_digits) {  // its three launches together, the gain in the second
+                st = timed(0, [&] { launch_stage(ctx, s); });
+                if (k == 0) per_step += qpr::kDigitLaunches;
             } else {
-                st = timed(2, [&] { qpr::launch_gain(s, ctx->ops, yin[s], w, ctx->stream); });
+                // the sparse stage forms the gain itself: there the gain kernel is timed beside it
+                // (as a stage without a stop decision, which the stage takes)
+                st = timed(2, [&] { qpr::launch_gain(ctx->d_H ? s : 3, ctx->ops, yin[s], w, ctx->stream); });
                 if (st == QPR_OK) st = timed(0, [&] { launch_stage(ctx, s); });
                 if (k == 0) per_step += 2;
             }
@@ -1582,7 +1596,7 @@ qpr_status qpr_profile_step(qpr_ctx *ctx, const void *rho, double dt, int64_t st
     }
     destroy();
     memset(out, 0, sizeof(*out));
-    out->product_ms = cnt[0] ? sum[0] / cnt[0] : 0.0;
+    out->product_ms = small ? sum[0] / (double)steps : cnt[0] ? sum[0] / cnt[0] : 0.0;
     out->epilogue_ms = cnt[1] ? sum[1] / cnt[1] : 0.0;
     out->gain_ms = cnt[2] ? sum[2] / cnt[2] : 0.0;
     out->refresh_ms = cnt[3] ? sum[3] / cnt[3] : 0.0;
