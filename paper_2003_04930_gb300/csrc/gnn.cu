@@ -771,8 +771,10 @@ qpr_status single_pass(qpr_gnn *g, const qpr::HostGraph &hg, const double *p, bo
     return QPR_OK;
 }
 
-// Nodes of a group at most (unless one graph has more): 250 MB of workspace.
-constexpr int kGroupNodes = 65536;
+// Workspace of a group at most (unless one graph needs more): some 70,000 nodes
+// in graphs of hundreds (4.7 KB a node), 2000 graphs of a few nodes (a block of
+// 128 rows of partial gradients, 104 KB, for the smallest).
+constexpr size_t kGroupBytes = (size_t)320 << 20;
 // The training set stays on the device up to this size; beyond it every group
 // is uploaded for its pass.
 constexpr size_t kResidentBytes = (size_t)2 << 30;
@@ -961,10 +963,11 @@ qpr_status qpr_gnn_train(qpr_gnn *g, int64_t count, const qpr_gnn_sample *sample
             const int64_t b1i = std::min<int64_t>(count, b0 + batch);
             for (int64_t k = b0; k < b1i;) {
                 std::vector<int64_t> ids;
-                int nodes = 0, maxn = 0;
-                for (; k < b1i && ids.size() < 4096 && (ids.empty() || nodes + hg[order[k]].n <= kGroupNodes); ++k) {
+                int maxn = 0;
+                size_t bytes = 0;
+                for (; k < b1i && (ids.empty() || bytes + ws_bytes(hg[order[k]].n) <= kGroupBytes); ++k) {
                     ids.push_back(order[k]);
-                    nodes += hg[order[k]].n;
+                    bytes += ws_bytes(hg[order[k]].n);
                     maxn = std::max(maxn, hg[order[k]].n);
                 }
                 const bool init = (int64_t)ids.size() == k - b0;  // the batch's first group
