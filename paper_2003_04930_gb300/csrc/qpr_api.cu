@@ -1194,7 +1194,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         if (digits) {
             cudaError_t e = cudaMalloc(&ctx->d_digits, qpr::digits_half_count(dplan, np) * 2);
             if (e == cudaSuccess) e = cudaMalloc(&ctx->d_digint, 3 * (size_t)np * sizeof(int));
-            if (e == cudaSuccess) e = cudaMalloc(&ctx->d_digx, (3 * plane + np) * sizeof(double));
+            if (e == cudaSuccess) e = cudaMalloc(&ctx->d_digx, qpr::digits_double_count(dplan, np) * sizeof(double));
             if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();
                 cudaFree(ctx->d_digits);

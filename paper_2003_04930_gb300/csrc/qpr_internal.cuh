@@ -258,16 +258,20 @@ struct DigitWork {
     int *ecol;            // [2 planes][np]: the exponent of the first digit's unit of a row of Y
     int *erow;            // np
     double *x;            // [H Re Y ; -H Im Y] without the diagonal of Y, 2 planes
-    const double *h;      // H, np x np
+    const void *hd;       // digit planes of H
+    const double *h;      // H, np x np (several digits)
+    int unit;             // one digit: H is the digits times 2^unit
     double *diag;         // the diagonal of the stage input, np
+    const double *hc;     // omega / 2 c, np
 };
 struct DigitMaps {
     CUtensorMap h, y;
 };
 // False if no digit width keeps the sums exact (stage_fp64.cu serves then).
 bool plan_digits(const HostOps &h, DigitPlan &p);
-// FP16 values of the digit planes; ints: 3 np, x: 3 np^2 + np.
+// FP16 values of the digit planes, doubles of x; ints: 3 np.
 size_t digits_half_count(const DigitPlan &p, int np);
+size_t digits_double_count(const DigitPlan &p, int np);
 cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *halves, int *ints, double *x, DigitWork *dw,
                         DigitMaps *maps);
 // The whole stage: digits of its input, product (with the gain and, at stage
@@ -374,7 +378,7 @@ int persist_grid(int np, int splits, int smem, int device, int *persist_smem, in
 cudaError_t set_persist_smem(int bytes);
 cudaError_t launch_cols_block(const DevOps &ops, const MixedWork &w, int steps, int grid, cudaStream_t s);
 // Kernel launches per RK4 step and per refresh of the mixed form.
-constexpr int kMixedLaunchesPerStep = 4;   // tile-pair sparse kernel (the dense one adds 4 gain kernels)
+constexpr int kMixedLaunchesPerStep = 4;   // tile-pair sparse kernel (the dense form: a product and an epilogue per stage)
 constexpr int kMixedLaunchesPerStepCols = 8;  // column-block form: SpMM (with the gain) and epilogue per stage
 inline int mixed_launches_per_refresh(const MixedWork &w) { return w.digits ? 6 : 4; }
 // Steady-state solves with adaptive_refresh: the longest window between

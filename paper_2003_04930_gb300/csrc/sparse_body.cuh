@@ -139,7 +139,7 @@ __device__ __forceinline__ void tile(const DevOps &ops, const Work &w, int I, in
                           STAGE == 1 && I == 0, red);
     spmm_pair(ops, yin, plane, I, J, diag, sX1, sX2, smem + 2 * TS * LDX);
     EpiIn<STAGE, NTHREADS> in;
-    in.load(ops, w, I, J);  // after the product: its registers are free (725 -> 615 us a step at N = 922)
+    in.load(ops, w, I, J, ops.c);  // after the product: its registers are free (725 -> 615 us a step at N = 922)
     stage_epilogue<STAGE, NTHREADS>(ops, w, I, J, diag, in, sX1, sX2, LDX, sg, red, pidx, first);
     __syncthreads();
 }

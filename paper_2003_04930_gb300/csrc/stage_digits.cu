@@ -53,6 +53,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "gain_body.cuh"
@@ -179,15 +180,18 @@ __global__ void __launch_bounds__(128) split_kernel(DevOps ops, Ctl *ctl, const 
     }
 }
 
-// Digits of the entries of H into the zeroed planes hd [sh][np][np], and the
-// entries themselves into the zeroed plane hf.
-__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd, double *hf) {
+// Digits of the entries of H into the zeroed planes hd [sh][np][np], and with
+// several digits the entries themselves into the zeroed plane hf; omega / 2 c
+// into hc.
+__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd, double *hf, double *hc) {
     const size_t plane = (size_t)ops.np * ops.np;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ops.np; i += gridDim.x * blockDim.x)
+        hc[i] = __dmul_rn(0.5 * ops.omega, ops.c[i]);
     for (int i = blockIdx.x; i < ops.n; i += gridDim.x)
         for (int q = ops.h_ptr[i] + threadIdx.x; q < ops.h_ptr[i + 1]; q += blockDim.x) {
             int16_t d[kMaxDigits];
             digits_of(ops.h_val[q], erow[i] - b * (sh - 1), sh, b, d);
-            hf[(size_t)i * ops.np + ops.h_col[q]] = ops.h_val[q];
+            if (sh > 1) hf[(size_t)i * ops.np + ops.h_col[q]] = ops.h_val[q];
             for (int s = 0; s < sh; ++s) hd[s * plane + (size_t)i * ops.np + ops.h_col[q]] = __short2half_rn(d[s]);
         }
 }
@@ -422,35 +426,51 @@ __global__ void __launch_bounds__(GT) digits_gemm_kernel(const __grid_constant__
 
 constexpr int LDX = 2 * kEpiTS + 1;
 constexpr int EPI_BYTES = 2 * kEpiTS * LDX * (int)sizeof(double);
-// 512 threads, two elements each: a stage takes 22.2, 26.5 and 41.1 us at N =
-// 200, 500 and 700 (unit weights); with 256 it took 22.8, 26.4 and 47.6.
+// 512 threads, two elements each: a stage takes 20.3, 26.2 and 39.2 us at N =
+// 100, 500 and 600 (unit weights), with 256 20.8, 26.0 and 44.9; from N = 1500
+// on it makes no difference (183 and 185 us).
 constexpr int ET = 512;
 
+// k 2^t from its digit k != 0, by integer instructions (exact); 0 from 0.
+__device__ __forceinline__ double from_digit(__half k, int t) {
+    const unsigned f = __float_as_uint(__half2float(k));
+    if ((f << 1) == 0) return 0.0;
+    return __hiloint2double((int)((f & 0x80000000u) | (((f & 0x7fffffffu) >> 3) + ((unsigned)(896 + t) << 20))), (int)(f << 29));
+}
+
 // The diagonal's part of A_ab - A_ba, which the product leaves out: H_ab (Y_bb -
-// Y_aa). H_ab in registers, the diagonal's entries of rows I and columns J in
-// shared memory (in registers too a stage took 0.3 us longer at N = 500).
+// Y_aa). H_ab in registers, from its one digit (ONE: no FP64 plane of H is
+// kept) or from the plane d.h; the diagonal's entries of rows I and columns J
+// in shared memory (in registers too a stage took 0.3 us longer at N = 500).
+template <bool ONE>
 struct DiagonalTerm {
     static constexpr int E = EpiIn<1, ET>::E;
-    double h[E];
+    typename std::conditional<ONE, __half, double>::type h[E];
     const double *sd;  // Y_aa of the 32 rows, then Y_bb of the 32 columns
+    int t;
 
     __device__ __forceinline__ void load(const DevOps &ops, const DigitWork &d, int I, int J, double *shared) {
+        t = d.unit;
 #pragma unroll
         for (int i = 0; i < E; ++i) {
             const int ga = I * kEpiTS + (threadIdx.x >> 5) + i * (ET / 32);
-            h[i] = __ldcg(d.h + (size_t)ga * ops.np + J * kEpiTS + (threadIdx.x & 31));
+            const size_t o = (size_t)ga * ops.np + J * kEpiTS + (threadIdx.x & 31);
+            if constexpr (ONE) h[i] = __ldcg(reinterpret_cast<const __half *>(d.hd) + o);
+            else h[i] = __ldcg(d.h + o);
         }
         if (threadIdx.x < 2 * kEpiTS)
             shared[threadIdx.x] = __ldcg(d.diag + (threadIdx.x < kEpiTS ? I : J) * kEpiTS + (threadIdx.x & 31));
         sd = shared;
     }
-    __device__ __forceinline__ double operator()(int i, double d) const {
+    __device__ __forceinline__ double rate(double, double hca, double hcb) const { return __dadd_rn(hca, hcb); }
+    __device__ __forceinline__ double difference(int i, double d) const {
         const double dy = __dsub_rn(sd[kEpiTS + (threadIdx.x & 31)], sd[(threadIdx.x >> 5) + i * (ET / 32)]);
-        return __fma_rn(h[i], dy, d);
+        if constexpr (ONE) return __fma_rn(from_digit(h[i], t), dy, d);
+        else return __fma_rn(h[i], dy, d);
     }
 };
 
-template <int STAGE>
+template <int STAGE, bool ONE>
 __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, DigitWork d) {
     extern __shared__ __align__(16) double sm[];
     __shared__ double red[ET / 32], sg[kEpiTS], s_diag[2 * kEpiTS];
@@ -461,8 +481,8 @@ __global__ void __launch_bounds__(ET) digits_epi_kernel(DevOps ops, Work w, Digi
     const size_t plane = (size_t)np * np;
     double *sX1 = sm, *sX2 = sm + kEpiTS * LDX;
     EpiIn<STAGE, ET> in;
-    in.load(ops, w, I, J);
-    DiagonalTerm dg;
+    in.load(ops, w, I, J, d.hc);
+    DiagonalTerm<ONE> dg;
     dg.load(ops, d, I, J, s_diag);
     tma::grid_dependency_wait();
     tma::launch_dependents();
@@ -523,7 +543,18 @@ void launch_t(const DevOps &ops, const Work &w, const DigitWork &d, const DigitM
         case 6: launch_sb<STAGE, 11, 6>(ops, w, d, m, s); break;
         default: launch_sb<STAGE, 13, 5>(ops, w, d, m, s); break;
     }
-    launch_dep(digits_epi_kernel<STAGE>, w.npairs, ET, (size_t)d.epi_smem, s, ops, w, d);
+    if (d.sh == 1) launch_dep(digits_epi_kernel<STAGE, true>, w.npairs, ET, (size_t)d.epi_smem, s, ops, w, d);
+    else launch_dep(digits_epi_kernel<STAGE, false>, w.npairs, ET, (size_t)d.epi_smem, s, ops, w, d);
+}
+
+template <bool ONE>
+cudaError_t init_epi(int smem) {
+    cudaError_t e = raise_smem_limit_t(digits_epi_kernel<0, ONE>, smem);
+    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<1, ONE>, smem);
+    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<2, ONE>, smem);
+    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<3, ONE>, smem);
+    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<4, ONE>, smem);
+    return e;
 }
 
 // The candidates: bits per digit and digits (S b >= 64).
@@ -588,6 +619,7 @@ bool plan_digits(const HostOps &h, DigitPlan &p) {
 }
 
 size_t digits_half_count(const DigitPlan &p, int np) { return (size_t)(p.sh + 2 * p.s) * np * np; }
+size_t digits_double_count(const DigitPlan &p, int np) { return (size_t)(p.sh > 1 ? 3 : 2) * np * np + 2 * (size_t)np; }
 
 cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *halves, int *ints, double *x, DigitWork *dw,
                         DigitMaps *maps) {
@@ -598,8 +630,12 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     dw->ecol = ints;
     dw->erow = ints + 2 * np;
     dw->x = x;
-    dw->h = x + 2 * plane;
-    dw->diag = x + 3 * plane;
+    dw->diag = x + 2 * plane;
+    dw->hd = hd;
+    double *hc = x + 2 * plane + np, *hf = hc + np;
+    dw->hc = hc;
+    dw->h = hf;
+    dw->unit = p.erow[0];
     dw->b = p.b;
     dw->s = p.s;
     dw->sh = p.sh;
@@ -611,7 +647,10 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     // product CTA at N = 500 (12.6 us against 4.5 for three). Where a CTA per
     // SM will do, each asks for more than half of an SM's shared memory.
     dw->epi_smem = ops.np / kEpiTS * (ops.np / kEpiTS + 1) / 2 <= sms ? 116 * 1024 : EPI_BYTES;
-    // rings: all of an SM when there is a tile per SM at most, else half of it
+    // rings: all of an SM when there is a tile per SM at most, else half of it,
+    // for two CTAs; with S >= 10 a CTA holds all of TMEM, so only one of them
+    // works, and at S = 11 and 13 the smallest rings are above the half (121
+    // and 137 KB)
     const int room = (tiles <= sms ? 200 : 96) * 1024;
     dw->ring_b = std::max(2, std::min(kMaxRing, room / (A_BYTES + p.s * B_ROW)));
     if (p.sh > 1) dw->ring_b = 2;
@@ -620,9 +659,9 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
     if (e != cudaSuccess) return e;
     e = cudaMemcpy(dw->erow, p.erow.data(), p.erow.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return e;
-    e = cudaMemset(x + 2 * plane, 0, plane * sizeof(double));
+    if (p.sh > 1) e = cudaMemset(hf, 0, plane * sizeof(double));
     if (e != cudaSuccess) return e;
-    split_h_kernel<<<std::min(ops.n, 4096), 128>>>(ops, p.b, p.sh, dw->erow, hd, x + 2 * plane);
+    split_h_kernel<<<std::min(ops.n, 4096), 128>>>(ops, p.b, p.sh, dw->erow, hd, hf, hc);
     e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return e;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
@@ -653,11 +692,7 @@ cudaError_t init_digits(const DevOps &ops, const DigitPlan &p, int sms, void *ha
         case 6: e = raise_smem_limit_t(digits_gemm_kernel<11, 6>, sm); break;
         default: e = raise_smem_limit_t(digits_gemm_kernel<13, 5>, sm); break;
     }
-    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<0>, dw->epi_smem);
-    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<1>, dw->epi_smem);
-    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<2>, dw->epi_smem);
-    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<3>, dw->epi_smem);
-    if (e == cudaSuccess) e = raise_smem_limit_t(digits_epi_kernel<4>, dw->epi_smem);
+    if (e == cudaSuccess) e = p.sh == 1 ? init_epi<true>(dw->epi_smem) : init_epi<false>(dw->epi_smem);
     return e;
 }
 

@@ -23,8 +23,8 @@
 //
 // What bounds it: the FP64 pipe (two operations a clock and SM) and, in a
 // small grid, the latency of its loads. So an element costs 10 FP64
-// operations a stage (15 to 17 with the running sum and a normalisation per
-// stage, and two divisions per thread before), and all of a thread's
+// operations a stage (11 in the digit products; 15 to 17 with the running sum
+// and a normalisation per stage, and two divisions per thread before), and all of a thread's
 // operands are loaded together by EpiIn::load: at N = 500 (136 pairs) 18.6 us
 // a launch before, 9.3 now (both with cold caches), 4.2 within a step.
 #pragma once
@@ -51,11 +51,12 @@ struct EpiIn {
     static constexpr int E = kEpiTS * kEpiTS / NT;
     double ir[E], ii[E], yr[E], yi[E], ca[E], cb, dt, scale;
 
-    __device__ __forceinline__ void load(const DevOps &ops, const Work &w, int I, int J) {
+    // c: ops.c, or what the product's form makes of it
+    __device__ __forceinline__ void load(const DevOps &ops, const Work &w, int I, int J, const double *c) {
         const size_t plane = (size_t)ops.np * ops.np;
         const double *yin = (STAGE <= 1) ? w.y : (STAGE == 3 ? w.yb : w.ya);
         const int b = threadIdx.x & 31;
-        cb = ops.c[J * kEpiTS + b];
+        cb = c[J * kEpiTS + b];
         dt = __ldcg(&w.ctl->dt);
         scale = (STAGE == 4) ? __ldcg(&w.ctl->scale) : 1.0;
 #pragma unroll
@@ -66,15 +67,20 @@ struct EpiIn {
             ii[i] = __ldcg(yin + plane + off);
             yr[i] = (STAGE >= 2) ? __ldcg(w.y + off) : ir[i];
             yi[i] = (STAGE >= 2) ? __ldcg(w.y + plane + off) : ii[i];
-            ca[i] = ops.c[ga];
+            ca[i] = c[ga];
         }
     }
 };
 
-// What the product left out of A_ab - A_ba of an element: nothing here, the
-// diagonal of the stage input in the digit products.
+// What differs between the products: the decay rate omega / 2 (c_a + c_b) from
+// what EpiIn holds for row and column (the digit products' epilogue holds
+// omega / 2 c, one operation less), and what the product left out of A_ab - A_ba of
+// element i (the digit products: the diagonal of the stage input).
 struct WholeProduct {
-    __device__ __forceinline__ double operator()(int, double d) const { return d; }
+    __device__ __forceinline__ double rate(double hom, double ca, double cb) const {
+        return __dmul_rn(hom, __dadd_rn(ca, cb));
+    }
+    __device__ __forceinline__ double difference(int, double d) const { return d; }
 };
 
 // Must be called by all NT threads of the CTA after the X tiles are complete
@@ -82,12 +88,12 @@ struct WholeProduct {
 // outputs, each by the one thread that reads that place.
 // g: the gain of rows I, read on diagonal pairs. pidx: slot of this tile
 // pair's residual partial; first: the tile pair that advances the step counter
-// at stage 4. rest(i, A_ab - A_ba) adds what the product left out.
+// at stage 4. form: WholeProduct or its like.
 template <int STAGE, int NT, typename P = WholeProduct>
 __device__ __forceinline__ void stage_epilogue(const DevOps &ops, const Work &w, int I, int J, bool diag,
                                                const EpiIn<STAGE, NT> &in, double *sX1, const double *sX2, int ldx,
                                                const double *g, double *red, int pidx, bool first,
-                                               const P &rest = P{}) {
+                                               const P &form = P{}) {
     constexpr int TS = kEpiTS, E = EpiIn<STAGE, NT>::E;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int np = ops.np;
@@ -110,9 +116,9 @@ __device__ __forceinline__ void stage_epilogue(const DevOps &ops, const Work &w,
         const size_t off = (size_t)ga * np + gb;
         const double Aab = sX1[a * ldx + b], nBab = sX1[a * ldx + TS + b];
         const double Aba = X2[b * ldx + a], nBba = X2[b * ldx + TS + a];
-        const double omhc = __dmul_rn(hom, __dadd_rn(in.ca[i], in.cb));  // the same for (b, a)
+        const double omhc = form.rate(hom, in.ca[i], in.cb);  // the same for (b, a)
         double kr = __fma_rn(-omhc, in.ir[i], __dmul_rn(-cm, __dadd_rn(nBab, nBba)));
-        const double ki = __fma_rn(-omhc, in.ii[i], __dmul_rn(-cm, rest(i, __dsub_rn(Aab, Aba))));
+        const double ki = __fma_rn(-omhc, in.ii[i], __dmul_rn(-cm, form.difference(i, __dsub_rn(Aab, Aba))));
         if (ga == gb) kr = __fma_rn(om, g[a], kr);
         if (STAGE <= 1) nrm = __fma_rn(kr, kr, __fma_rn(ki, ki, nrm));
         double o0 = kr, o1 = ki;

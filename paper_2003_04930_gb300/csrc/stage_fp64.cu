@@ -151,7 +151,7 @@ stage_fp64_kernel(DevOps ops, Work w) {
     double *sX1 = smem;                 // X_IJ: [TS][LDX], columns 0..TS-1 real, TS..2TS-1 imaginary
     double *sX2 = smem + TS * LDX;      // X_JI
     EpiIn<STAGE, NTHREADS> in;
-    in.load(ops, w, I, J);
+    in.load(ops, w, I, J, ops.c);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
