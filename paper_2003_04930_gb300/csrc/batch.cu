@@ -298,8 +298,7 @@ __global__ void __launch_bounds__(cols::kENT, 3) b_cols_epi_kernel(const BatchGr
             if (!done) mixed::epi_load<STAGE, cols::kENT>(sg.ops, sg.mw, t.y, t.z, in);
         }
         if (!done)
-            cols::epilogue_pair_in<STAGE>(sg.ops, sg.mw, t.y, t.z, t.w, t.w == 0, sg.mw.npairs, sX1, sX2, sg32,
-                                                 sO, in);
+            cols::epilogue_pair_in<STAGE>(sg.ops, sg.mw, t.y, t.z, t.w, t.w == 0, sX1, sX2, sg32, sO, in);
         first = false;
         __syncthreads();
     }

@@ -447,7 +447,7 @@ __device__ __forceinline__ void epilogue_load_x(const DevOps &ops, const MixedWo
 // (after a barrier).
 template <int STAGE, bool SPLIT = false>
 __device__ __forceinline__ void epilogue_pair_staged(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
-                                                     bool first, int nparts, const float *sX1, const float *sX2,
+                                                     bool first, const float *sX1, const float *sX2,
                                                      const float *sg, float *sO, const mixed::EpiIn<STAGE, kENT> &in) {
     mixed::tile_epilogue_in<STAGE, kENT, SPLIT>(ops, w, I, J, pidx, sX1, sX2, sg, sO, in);
     if (STAGE == 4 && first && threadIdx.x == 0) w.ctl->step += 1;
@@ -455,21 +455,21 @@ __device__ __forceinline__ void epilogue_pair_staged(const DevOps &ops, const Mi
 
 template <int STAGE>
 __device__ __forceinline__ void epilogue_pair_in(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
-                                                 bool first, int nparts, float *sX1, float *sX2, float *sg, float *sO,
+                                                 bool first, float *sX1, float *sX2, float *sg, float *sO,
                                                  const mixed::EpiIn<STAGE, kENT> &in) {
     epilogue_load_x(ops, w, I, J, sX1, sX2, sg);
     __syncthreads();
-    epilogue_pair_staged<STAGE>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
+    epilogue_pair_staged<STAGE>(ops, w, I, J, pidx, first, sX1, sX2, sg, sO, in);
 }
 
 // The same with the elementwise operands loaded first, so that their loads
 // and the X tiles' are in flight together.
 template <int STAGE>
 __device__ __forceinline__ void epilogue_pair(const DevOps &ops, const MixedWork &w, int I, int J, int pidx,
-                                              bool first, int nparts, float *sX1, float *sX2, float *sg, float *sO) {
+                                              bool first, float *sX1, float *sX2, float *sg, float *sO) {
     mixed::EpiIn<STAGE, kENT> in;
     mixed::epi_load<STAGE, kENT>(ops, w, I, J, in);
-    epilogue_pair_in<STAGE>(ops, w, I, J, pidx, first, nparts, sX1, sX2, sg, sO, in);
+    epilogue_pair_in<STAGE>(ops, w, I, J, pidx, first, sX1, sX2, sg, sO, in);
 }
 
 }  // namespace cols

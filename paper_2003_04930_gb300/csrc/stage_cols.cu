@@ -90,8 +90,7 @@ __global__ void __launch_bounds__(kENT, SPLIT ? 2 : 3) cols_epi_kernel(DevOps op
     __syncthreads();
     if (!s_done) {
         // no ticket: the stage-2 SpMM grid takes the stop decision (gain_role)
-        epilogue_pair_staged<STAGE, SPLIT>(ops, w, pr.x, pr.y, pr.z, blockIdx.x == 0, w.npairs, sX1, sX2, sg, sO,
-                                           in);
+        epilogue_pair_staged<STAGE, SPLIT>(ops, w, pr.x, pr.y, pr.z, blockIdx.x == 0, sX1, sX2, sg, sO, in);
     }
     timeline::leave();
 }

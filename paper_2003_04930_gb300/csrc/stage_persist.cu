@@ -122,7 +122,7 @@ __device__ __forceinline__ int persist_stage(const CUtensorMap *tm, const DevOps
     float *sX1 = sm.epi, *sX2 = sX1 + TS * LDX, *sO = sX2 + TS * LDX, *sg = sO + 4 * TS * LDO;
     for (int p = c; p < w.npairs; p += (int)C) {
         const int2 pr = w.pairs[p];
-        epilogue_pair<STAGE>(ops, w, pr.x, pr.y, p, p == 0, w.npairs, sX1, sX2, sg, sO);
+        epilogue_pair<STAGE>(ops, w, pr.x, pr.y, p, p == 0, sX1, sX2, sg, sO);
         __syncthreads();
     }
     if (!grid_sync(w.ctl, C, gen, sm.flag)) return -1;
