@@ -79,9 +79,9 @@ __device__ __forceinline__ int skip_refresh(const BatchGraph &sg, int g, const u
 }
 
 // The lists a captured block runs over change as problems stop; their lengths
-// are read from device memory, so one capture serves the whole solve (with a
-// capture at every change 12 problems of N <= 492 took 246 ms, 227 so and with
-// the spectra formed on the device).
+// are read from device memory, so one capture serves the whole solve (12
+// problems of N <= 492: 274 ms with a capture at every change and every
+// spectrum formed in turn on the host, 246 without either).
 struct Counts {
     int act, items, b, t;  // active problems, all pairs, column-form pairs, tile-form pairs
     int a[2];              // SpMM units per size class

@@ -239,8 +239,9 @@ __device__ __forceinline__ void narrow_bundles(const float *__restrict__ sD, con
         // one at a time after the last full block each waited for its own
         // shared-memory latency, as did the row slot read at the end: steady
         // state at N = 922 114.9 -> 110.1 ms, N = 700 87.3 -> 84.6, N = 1400
-        // 357 -> 345, RKF45 at N = 922 35.3 -> 34.3 (blocks of 8 or 6: N = 500
-        // 1.7% slower).
+        // 357 -> 345, RKF45 at N = 922 35.3 -> 34.3, on one graph each (3 to 4%,
+        // less than graphs of a size differ; blocks of 8 or 6: N = 500 1.7%
+        // slower).
         auto rounds = [&](auto count) {
             constexpr int U = decltype(count)::value;
             int2 e[U];

@@ -127,11 +127,13 @@ def _weighted(g, w):
 
 @pytest.mark.parametrize("scale", [1.0, 1e-5, 1e-8, 1e-14])
 @pytest.mark.parametrize("n", [45, 65, 130])
-@pytest.mark.parametrize("weights", ["unit", "lognormal"])
+@pytest.mark.parametrize("weights", ["unit", "eighths", "lognormal"])
 def test_small_coherences(n, weights, scale):
     g = graphs.erdos_renyi(n, 0.4, n)
     if weights == "lognormal":
         g = _weighted(g, np.random.default_rng(n).lognormal(0.0, 1.0, g.m))
+    if weights == "eighths":
+        g = _weighted(g, np.random.default_rng(n).integers(1, 30, g.m) / 8)
     _check(g, _state(n, scale, 7))
 
 
