@@ -108,8 +108,8 @@ __global__ void __cluster_dims__(kPrCtas, 1, 1) __launch_bounds__(kPrT, 1)
 pagerank_cluster_kernel(const PrJob *__restrict__ jobs, PrJob one, int iters, double tol, long long max_iter,
                         double *state) {
     extern __shared__ __align__(16) double sm[];
-    // the CTAs' parts of the L1 change, one copy for every other check: a limit
-    // of 8 m + 1 iterations makes two checks follow each other with one barrier
+    // the CTAs' parts of the L1 change, one copy for every other iteration: a
+    // limit of 8 m + 1 makes two checks follow each other with one barrier
     // between, and a CTA may still read the first while a peer stores the second
     __shared__ double s_part[4], s_dang, s_delta[2][kPrCtas], red[32];
     const PrJob g = jobs ? jobs[blockIdx.y] : one;
@@ -132,7 +132,7 @@ pagerank_cluster_kernel(const PrJob *__restrict__ jobs, PrJob one, int iters, do
     const double tele = (1.0 - g.alpha) * inv_nm1;
     __syncthreads();
     pr_barrier();  // the cluster's CTAs run, and have read the state
-    int cur = 0, chk = 0;
+    int cur = 0;
     bool stopped = false;
     double delta = 0.0;
     for (int k = 0; k < iters && !stopped; ++k) {
@@ -187,14 +187,13 @@ pagerank_cluster_kernel(const PrJob *__restrict__ jobs, PrJob one, int iters, do
         }
         if (check) {
             dl = block_sum(dl, red);
-            if (tid < kPrCtas) pr_store(pr_remote(&s_delta[chk][cta], tid), dl);
+            if (tid < kPrCtas) pr_store(pr_remote(&s_delta[cur][cta], tid), dl);
         }
         pr_barrier();
         cur = 1 - cur;
         if (check) {
             delta = 0.0;
-            for (int c = 0; c < kPrCtas; ++c) delta += s_delta[chk][c];
-            chk ^= 1;
+            for (int c = 0; c < kPrCtas; ++c) delta += s_delta[1 - cur][c];
             stopped = !(delta >= tol) || it >= max_iter;  // the same in every CTA
         }
     }
