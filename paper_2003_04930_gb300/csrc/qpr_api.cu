@@ -575,12 +575,15 @@ double estimate_spread(const HostOps &h) {
     return bounded_spread(h, fabs(l2) * 1.02 + 1e-12);
 }
 
-// A thread for every 4000 nonzeros (about 2 ms of power iteration), 16 at most.
+// A thread for every 1000 nonzeros (about 0.5 ms of power iteration), 16 at
+// most: a batch to 1e-3 of 5 graphs of N <= 200 takes 41.7 ms, of 40 of N <= 469
+// 228.9 (one for every 4000: 42.5 and 228.9; in clusters on the device from 500
+// nonzeros on: 44.1 and 235.8).
 bool estimate_spreads(const std::vector<HostOps> &h, const std::vector<size_t> &which, std::vector<double> &out) {
     size_t nnz = 0;
     for (size_t g : which) nnz += h[g].hval.size();
     const size_t cpus = std::max(1u, std::thread::hardware_concurrency());
-    const size_t want = std::min({which.size(), nnz / 4000 + 1, cpus, (size_t)16});
+    const size_t want = std::min({which.size(), nnz / 1000 + 1, cpus, (size_t)16});
     std::atomic<size_t> next{0};
     std::atomic<bool> ok{true};
     auto run = [&] {
@@ -1188,7 +1191,7 @@ qpr_status qpr_create(qpr_ctx **out, int64_t n, int64_t m, const int64_t *src, c
         // the product on the tensor cores by exact digits where a plan keeps
         // the sums exact and its planes fit beside everything else; else the
         // FP64 tensor kernel and its dense H (N = 500, unit weights: 616 us a
-        // stage there, 27 us here; N = 922, lognormal weights: 4.2 and 0.36 ms)
+        // stage there, 26 us here; N = 922, lognormal weights: 4.2 and 0.36 ms)
         qpr::DigitPlan dplan;
         bool digits = qpr::plan_digits(hops, dplan);
         if (digits) {

@@ -4,11 +4,12 @@
 //
 // On the host this was most of a context's set-up (800 sweeps over the
 // nonzeros: qpr_create 10.3 ms at N = 922, 196 ms at N = 900 with 394 nonzeros
-// a row; 6.4 and 34 with this). What bounds it here is the chain of a product: a row's FP64 sum and one cluster barrier, 3.7 us at N = 300 and 4.2 at 922. So the
-// vector stays in every CTA's shared memory (two buffers, entries written
-// through distributed shared memory), four lanes sum a row (a warp one of more
-// than kLong entries), the vector is rescaled by its norm only at every eighth
-// product, and the Rayleigh quotient is formed at the last one.
+// a row; 6.4 and 34 with this). What bounds it here is the chain of a product:
+// a row's FP64 sum and one cluster barrier, 3.7 us at N = 300 and 4.2 at 922.
+// So the vector stays in every CTA's shared memory (two buffers, entries
+// written through distributed shared memory), four lanes sum a row (a warp one
+// of more than kLong entries), the vector is rescaled by its norm only at every
+// eighth product, and the Rayleigh quotient is formed at the last one.
 #include <math.h>
 
 #include <algorithm>

@@ -6,7 +6,7 @@
 // Why: FP64 runs at 1.04 TFLOP/s on this part, FP16 with FP32 accumulation at
 // about 1900. The FP64 tensor instruction (stage_fp64.cu) took 616 us per
 // stage at N = 500 (4.2 ms at N = 922), one 32 x 32 tile pair per CTA; this
-// form takes 27 us at N = 500 with unit weights and 363 us at N = 922 with
+// form takes 26 us at N = 500 with unit weights and 362 us at N = 922 with
 // lognormal ones. Here every entry off the diagonal is written as
 //     Y_jk = 2^(ec_j) sum_s y_s(j, k) 2^(-b s),   s < S,  |y_s| <= 2^(b-1),
 // with integers y_s (exact in FP16) and ec_j from the largest entry of row j
@@ -24,7 +24,7 @@
 // to these largest entries: an entry of Y further below its column's largest
 // than S b - 53 bits (11 to 19) enters with fewer than FP64's 53 bits. The
 // diagonal, which is what towers over a column in a state with small
-// coherences, therefore stays out of the product and is added exactly by the
+// coherences, therefore stays out of the product and is added in FP64 by the
 // epilogue as H_ab (Y_bb - Y_aa) (DiagonalTerm): with it in the product,
 // entries of pairs that are not linked were off by up to 1e-13 of their terms
 // with coherences of 1e-5 / N and 1e-10 with 1e-8 / N, now 1e-16 (CPU model, N =
@@ -183,7 +183,8 @@ __global__ void __launch_bounds__(128) split_kernel(DevOps ops, Ctl *ctl, const 
 // Digits of the entries of H into the zeroed planes hd [sh][np][np], and with
 // several digits the entries themselves into the zeroed plane hf; omega / 2 c
 // into hc.
-__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd, double *hf, double *hc) {
+__global__ void split_h_kernel(DevOps ops, int b, int sh, const int *__restrict__ erow, __half *hd, double *hf,
+                               double *hc) {
     const size_t plane = (size_t)ops.np * ops.np;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ops.np; i += gridDim.x * blockDim.x)
         hc[i] = __dmul_rn(0.5 * ops.omega, ops.c[i]);
@@ -435,7 +436,8 @@ constexpr int ET = 512;
 __device__ __forceinline__ double from_digit(__half k, int t) {
     const unsigned f = __float_as_uint(__half2float(k));
     if ((f << 1) == 0) return 0.0;
-    return __hiloint2double((int)((f & 0x80000000u) | (((f & 0x7fffffffu) >> 3) + ((unsigned)(896 + t) << 20))), (int)(f << 29));
+    const unsigned hi = ((f & 0x7fffffffu) >> 3) + ((unsigned)(896 + t) << 20);  // the exponent rebiased, plus t
+    return __hiloint2double((int)((f & 0x80000000u) | hi), (int)(f << 29));
 }
 
 // The diagonal's part of A_ab - A_ba, which the product leaves out: H_ab (Y_bb -
